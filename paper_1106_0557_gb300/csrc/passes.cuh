@@ -36,6 +36,8 @@
 // run a persistent grid on the lengths that keep their twiddles in
 // registers).
 #pragma once
+#include <type_traits>
+
 #include "fft_engine.cuh"
 #include "launch.h"
 #include "tma.cuh"
@@ -332,6 +334,24 @@ struct ZCfg {
     static_assert(G_BLK % 16 == 0, "bulk copies move multiples of 16 bytes");
     static_assert(E % 2 == 0, "the z pass splits a thread's points at L/2");
 };
+
+// kx tile of the i-th tile of line pair pr (ntx tiles per pair).  The walk
+// of a persistent CTA advances by the grid size, which shares factors with
+// ntx (152 and 32 at 256^3), so with xt = i the same few CTAs meet every
+// tile that holds the packed column (xt = 0), whose partner exchange and
+// spectrum loads make it longer than the others, and end last: the SMs were
+// busy for 88 % of the z pass at FP32 256^3.  Rotating the tiles of each pair
+// spreads them over all CTAs: 200.0 -> 187.0 us at 256^3, 69.9 -> 58.1 us at
+// 64 x 256 x 256 (ntx = 8 divides 152), FP64 780 -> 760 us at 128^3.  Float
+// pairs keep xt = i: their tiles are all arithmetic, and their registers are
+// full (the two index operations cost 4 % at 512 points, 17 % at 384).
+template <typename T>
+__device__ __forceinline__ int z_rotate(int i, int pr, int ntx)
+{
+    if constexpr (std::is_same<T, df64>::value) return i;
+    const int r = i + (pr + (pr >> 2)) % ntx;
+    return r >= ntx ? r - ntx : r;
+}
 
 // Layout of the Green's spectrum read by the z pass: [ky'][kx tile][kz'][TX]
 // with ky' <= My/2, kz' <= Mz/2 and kx = tile * TX + c (padded with zeros
@@ -1096,7 +1116,7 @@ k_z_convolve(const __grid_constant__ CUtensorMap tmW, Cx<T> *__restrict__ W, con
     // copies of a tile into the input set and spectrum set `set`, issued by
     // thread 0
     auto issue = [&](int tile, int set, uint32_t extra) {
-        const int pr = tile / ntx, xt = tile - pr * ntx;
+        const int pr = tile / ntx, xt = z_rotate<T>(tile - pr * ntx, pr, ntx);
         const int ky1 = pr == 0 ? My / 2 : My - pr;
         mbar_arrive_expect_tx(&bar[0], (uint32_t)(C::IN_SET + (pr == 0 ? 2 : 1) * C::G_BLK) + extra);
 #pragma unroll
@@ -1130,7 +1150,7 @@ k_z_convolve(const __grid_constant__ CUtensorMap tmW, Cx<T> *__restrict__ W, con
             ok = false;
             break;
         }
-        const int pr = tile / ntx, xt = tile - pr * ntx;
+        const int pr = tile / ntx, xt = z_rotate<T>(tile - pr * ntx, pr, ntx);
         // line group 1 staged one row later with SHIFT (its row 0 is plane -1)
         const Cx<T> *sin = reinterpret_cast<const Cx<T> *>(s_in + g * C::IN_GROUP) + (C::SHIFT && g ? TX : 0);
         const T *sg = s_g + ((size_t)set * 2 + (pr == 0 ? g : 0)) * C::GBLK;
@@ -1202,7 +1222,7 @@ k_z_convolve_pairs(const __grid_constant__ CUtensorMap tmW, Cx<T> *__restrict__ 
     // thread 0 issues; n_in / n_g count the phases issued on each barrier
     int n_in = 0, n_g = 0;
     auto issue_in = [&](int pair, uint32_t extra) {
-        const int pr = pair / npx, xt0 = 2 * (pair - pr * npx);
+        const int pr = pair / npx, xt0 = 2 * z_rotate<T>(pair - pr * npx, pr, npx);
         const int ky1 = pr == 0 ? My / 2 : My - pr;
         mbar_arrive_expect_tx(&bar[0], (uint32_t)C::PIN_SET + extra);
 #pragma unroll
@@ -1220,7 +1240,7 @@ k_z_convolve_pairs(const __grid_constant__ CUtensorMap tmW, Cx<T> *__restrict__ 
         ++n_in;
     };
     auto issue_g = [&](int pair) {
-        const int pr = pair / npx, xt0 = 2 * (pair - pr * npx);
+        const int pr = pair / npx, xt0 = 2 * z_rotate<T>(pair - pr * npx, pr, npx);
         const uint32_t bytes = (uint32_t)((ntx - xt0 < 2 ? 1 : 2) * C::G_BLK);
         mbar_arrive_expect_tx(&bar[1], (pr == 0 ? 2u : 1u) * bytes);
         bulk_load(s_g, G + lay.block(pr, xt0), bytes, &bar[1]);
@@ -1244,7 +1264,7 @@ k_z_convolve_pairs(const __grid_constant__ CUtensorMap tmW, Cx<T> *__restrict__ 
             break;
         }
         in_done = true;
-        const int pr = pair / npx, xt0 = 2 * (pair - pr * npx);
+        const int pr = pair / npx, xt0 = 2 * z_rotate<T>(pair - pr * npx, pr, npx);
         const int nsub = ntx - xt0 < 2 ? 1 : 2;
         for (int s = 0; s < nsub; ++s) {
             const bool last = s == nsub - 1;
