@@ -671,7 +671,8 @@ k_x_forward(const In<T> *__restrict__ src, Cx<T> *__restrict__ W, const Cx<T> *_
     if constexpr (C::TWR_F) {
         RowTwiddles<true, T, L, SH> twr;
         twr.load(tw, t);
-        for (int64_t r0 = (int64_t)blockIdx.x * C::NL; r0 < nrows; r0 += (int64_t)gridDim.x * C::NL) {
+        grid_wait();
+            for (int64_t r0 = (int64_t)blockIdx.x * C::NL; r0 < nrows; r0 += (int64_t)gridDim.x * C::NL) {
             const int64_t row = r0 + l;  // row = z * Ny + y
             const bool active = row < nrows;
             x_forward_row<T, L, true, SH>(src, W, tw, rtw, Nx, Ny, My, active ? row : 0, active, line, t, zsh, twr);
@@ -682,10 +683,11 @@ k_x_forward(const In<T> *__restrict__ src, Cx<T> *__restrict__ W, const Cx<T> *_
             }
         }
     } else {
+        grid_wait();
         const int64_t row = (int64_t)blockIdx.x * C::NL + l;
         const bool active = row < nrows;
         x_forward_row<T, L, false, SH>(src, W, tw, rtw, Nx, Ny, My, active ? row : 0, active, line, t, zsh);
-    }
+        }
 }
 
 template <typename T, int L>
@@ -700,17 +702,19 @@ k_x_inverse(const Cx<T> *__restrict__ W, In<T> *__restrict__ phi, const Cx<T> *_
     if constexpr (C::TWR_I) {
         RowTwiddles<true, T, L> twr;
         twr.load(tw, t);
-        for (int64_t r0 = (int64_t)blockIdx.x * C::NL; r0 < nrows; r0 += (int64_t)gridDim.x * C::NL) {
+        grid_wait();
+            for (int64_t r0 = (int64_t)blockIdx.x * C::NL; r0 < nrows; r0 += (int64_t)gridDim.x * C::NL) {
             const int64_t row = r0 + l;
             const bool active = row < nrows;
             x_inverse_row<T, L, false, true>(W, phi, tw, rtw, Nx, Ny, My, active ? row : 0, active, line, t, zsh,
                                              twr);
         }
     } else {
+        grid_wait();
         const int64_t row = (int64_t)blockIdx.x * C::NL + l;
         const bool active = row < nrows;
         x_inverse_row<T, L>(W, phi, tw, rtw, Nx, Ny, My, active ? row : 0, active, line, t, zsh);
-    }
+        }
 }
 
 // ---------------------------------------------------------------------
@@ -725,6 +729,7 @@ k_y_forward(Cx<T> *__restrict__ W, const Cx<T> *__restrict__ tw, int Ny, int Kx,
 {
     using C = ColCfg<T, L, NARROW>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    grid_wait();
     y_forward_tile<T, L, C::TX, false, BLK>(W, tw, Ny, Kx, blockIdx.y, blockIdx.x * C::TX,
                                             reinterpret_cast<Cx<T> *>(smem_raw), threadIdx.x % C::TX,
                                             threadIdx.x / C::TX, nullptr, zsh);
@@ -736,6 +741,7 @@ k_y_inverse(Cx<T> *__restrict__ W, const Cx<T> *__restrict__ tw, int Ny, int Kx,
 {
     using C = ColCfg<T, L, NARROW>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    grid_wait();
     y_inverse_tile<T, L, C::TX, BLK>(W, tw, Ny, Kx, blockIdx.y, blockIdx.x * C::TX,
                                      reinterpret_cast<Cx<T> *>(smem_raw), threadIdx.x % C::TX, threadIdx.x / C::TX,
                                      nullptr, zsh);
@@ -862,6 +868,7 @@ k_y_pass(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtens
     const int c = tid % TX, t = tid / TX;
     const int ntx = (Kx + TX - 1) / TX;
     if (smem_addr(ysmem) & 127u) {
+        grid_wait();
         if (tid == 0 && status) atomicOr(status, 2u);
         return;
     }
@@ -897,6 +904,7 @@ k_y_pass(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtens
     };
     int tile = blockIdx.x, it = 0;
     bool ok = true;
+    grid_wait();
     if (tid == 0 && tile < ntiles) issue(tile, 0);
     for (; tile < ntiles; tile += gridDim.x, ++it) {
         const int next = tile + gridDim.x;
@@ -1098,6 +1106,7 @@ k_z_convolve(const __grid_constant__ CUtensorMap tmW, Cx<T> *__restrict__ W, con
 
     // tensor copies need 128-byte aligned destinations (uniform per CTA)
     if (smem_addr(zsmem) & 127u) {
+        grid_wait();
         if (tid == 0 && status) atomicOr(status, 2u);
         return;
     }
@@ -1138,6 +1147,7 @@ k_z_convolve(const __grid_constant__ CUtensorMap tmW, Cx<T> *__restrict__ W, con
     bool ok = true;
     // test_extra_tx is a test hook: bytes the first tile's barrier expects
     // beyond what its copies deliver, so that its wait runs out (normally 0)
+    grid_wait();
     if (tid == 0 && tile < ntiles) issue(tile, 0, test_extra_tx);
     for (; tile < ntiles; tile += gridDim.x, ++it) {
         const int next = tile + gridDim.x;
@@ -1203,6 +1213,7 @@ k_z_convolve_pairs(const __grid_constant__ CUtensorMap tmW, Cx<T> *__restrict__ 
     const ZSpecLayout lay{TX, ntx, Lh + 1, C::GBLK};
 
     if (smem_addr(zsmem) & 127u) {
+        grid_wait();
         if (tid == 0 && status) atomicOr(status, 2u);
         return;
     }
@@ -1252,6 +1263,7 @@ k_z_convolve_pairs(const __grid_constant__ CUtensorMap tmW, Cx<T> *__restrict__ 
     twr.load(tw, t);
     int pair = blockIdx.x, it = 0;
     bool ok = true, in_done = false;
+    grid_wait();
     if (tid == 0 && pair < npairs) {
         issue_in(pair, test_extra_tx);
         issue_g(pair);

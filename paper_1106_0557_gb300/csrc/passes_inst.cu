@@ -35,6 +35,35 @@ static cudaError_t ensure_smem(F *func, size_t bytes, std::atomic<uint64_t> &don
     return e;
 }
 
+// Launch with the programmatic-serialization attribute: the launch is
+// processed while the stream's previous kernel still runs, its CTAs start as
+// that kernel's last ones leave, and each waits in grid_wait() before it
+// touches the previous results.  Without it every pass of a small solve paid
+// about 2 us between kernels: solves back to back in one stream took 24.9 us
+// at FP32 64^3 (17.2 now), 28.0 at 100 x 70 x 30 (17.7), 70.0 at 128^3 (57.0),
+// 416 at 256^3 (404.5).  The kernels do not trigger their successors early
+// (griddepcontrol.launch_dependents): CTAs that sit waiting hold the SM room
+// that solves on other streams could use (64 grids on eight streams 942-960
+// us with triggers at the start or end of each CTA, 922-930 without, 935
+// before).
+template <typename... K, typename... A>
+static cudaError_t launch_pass(void (*kernel)(K...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, K(args)...);
+    count_launch();
+    return e;
+}
+
 #define ISOFFT_ROW_LENGTHS(X) \
     X(16) X(24) X(32) X(48) X(64) X(96) X(128) X(192) X(256) X(384) X(512) X(768) X(1152)
 #define ISOFFT_COL_LENGTHS(X) \
@@ -98,10 +127,8 @@ static cudaError_t run_x_forward(const In<T> *src, void *W, const void *tw, cons
     if (e != cudaSuccess) return e;
     const unsigned grid =
         row_grid(nrows, C::NL, C::TWR_F ? resident_ctas(k_x_forward<T, L>, C::THREADS, C::SMEM, resident) : 0);
-    k_x_forward<T, L><<<grid, C::THREADS, C::SMEM, st>>>(src, (Cx<T> *)W, (const Cx<T> *)tw,
-                                                        (const Cx<T> *)rtw, Nx, Ny, My, nrows, zsh);
-    count_launch();
-    return cudaGetLastError();
+    return launch_pass(k_x_forward<T, L>, dim3(grid), C::THREADS, C::SMEM, st, src, (Cx<T> *)W, (const Cx<T> *)tw,
+                       (const Cx<T> *)rtw, Nx, Ny, My, nrows, zsh);
 }
 template <typename T, int L>
 static cudaError_t run_x_inverse(const void *W, In<T> *phi, const void *tw, const void *rtw, int Nx, int Ny,
@@ -115,10 +142,8 @@ static cudaError_t run_x_inverse(const void *W, In<T> *phi, const void *tw, cons
     if (e != cudaSuccess) return e;
     const unsigned grid =
         row_grid(nrows, C::NL, C::TWR_I ? resident_ctas(k_x_inverse<T, L>, C::THREADS, C::SMEM, resident) : 0);
-    k_x_inverse<T, L><<<grid, C::THREADS, C::SMEM, st>>>((const Cx<T> *)W, phi, (const Cx<T> *)tw,
-                                                        (const Cx<T> *)rtw, Nx, Ny, My, nrows, zsh);
-    count_launch();
-    return cudaGetLastError();
+    return launch_pass(k_x_inverse<T, L>, dim3(grid), C::THREADS, C::SMEM, st, (const Cx<T> *)W, phi,
+                       (const Cx<T> *)tw, (const Cx<T> *)rtw, Nx, Ny, My, nrows, zsh);
 }
 
 template <typename R_>
@@ -164,9 +189,7 @@ static cudaError_t run_y_tile(void *W, const void *tw, int Ny, int Kx, int Nz, i
     cudaError_t e = ensure_smem(k, C::SMEM, zsh ? doneb : done0);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)((Kx + C::TX - 1) / C::TX), (unsigned)Nz);
-    k<<<grid, C::THREADS, C::SMEM, st>>>((Cx<T> *)W, (const Cx<T> *)tw, Ny, Kx, zsh);
-    count_launch();
-    return cudaGetLastError();
+    return launch_pass(k, dim3(grid), C::THREADS, C::SMEM, st, (Cx<T> *)W, (const Cx<T> *)tw, Ny, Kx, zsh);
 }
 template <typename T, int L, bool FWD>
 static cudaError_t run_y_stream(void *W, const void *tw, int Ny, int Kx, int Nz, int zsh, unsigned *status,
@@ -216,9 +239,8 @@ static cudaError_t run_y_stream(void *W, const void *tw, int Ny, int Kx, int Nz,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
     }
-    k<<<grid, C::THREADS, SMEM, st>>>(map, omap, (Cx<T> *)W, (const Cx<T> *)tw, Ny, Kx, ntiles, status, zsh);
-    count_launch();
-    return cudaGetLastError();
+    return launch_pass(k, dim3(grid), C::THREADS, SMEM, st, map, omap, (Cx<T> *)W, (const Cx<T> *)tw, Ny, Kx,
+                       ntiles, status, zsh);
 }
 template <typename T, int L, bool FWD>
 static cudaError_t run_y(void *W, const void *tw, int Ny, int Kx, int Nz, int zsh, unsigned *status, int variant,
@@ -317,10 +339,8 @@ static cudaError_t run_z(void *W, const void *tw, const T *G, const T *Gs, T gsc
                zsh ? box4 : box3, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
-    kernel<<<grid, C::THREADS, C::SMEM, st>>>(map, (Cx<T> *)W, (const Cx<T> *)tw, G, Gs, gscale, Nz, My, Kx, units,
-                                             status, test_extra_tx);
-    count_launch();
-    return cudaGetLastError();
+    return launch_pass(kernel, dim3(grid), C::THREADS, C::SMEM, st, map, (Cx<T> *)W, (const Cx<T> *)tw, G, Gs, gscale,
+                       Nz, My, Kx, units, status, test_extra_tx);
 }
 template <typename R_>
 cudaError_t launch_z_convolve(int L, void *W, const void *tw, const R_ *G, const R_ *Gs, R_ gscale,

@@ -124,6 +124,11 @@ __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wa
 // this thread's shared-memory writes become visible to the tensor copies
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
 
+// Programmatic dependent launch: returns when every earlier kernel of the
+// stream has finished and its writes are visible (at once if this kernel was
+// launched without the attribute).
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+
 // Time limit of one wait for a tile's copies (they normally land within
 // microseconds).
 constexpr uint64_t kCopyWaitNs = 2000000000ull;
