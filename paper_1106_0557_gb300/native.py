@@ -156,8 +156,9 @@ def ipf_estimate_bytes(n, h, dtype="f32"):
 
 
 def ipf_solve(plan, d_src, d_phi, stream=0):
-    _check(lib().ipf_solve(ctypes.c_void_p(plan), ctypes.c_void_p(int(d_src)), ctypes.c_void_p(int(d_phi)),
-                           ctypes.c_void_p(int(stream))), "ipf_solve")
+    rc = lib().ipf_solve(plan, int(d_src), int(d_phi), int(stream))  # argtypes convert the addresses
+    if rc != IPF_OK:
+        raise IsofftError(rc, "ipf_solve")
 
 
 def ipf_solve_host(plan, h_src, h_phi, stream=0):

@@ -14,10 +14,18 @@ _TORCH = {"f32": torch.float32, "f64": torch.float64, "df64": torch.float64}
 _NUMPY = {"f32": np.float32, "f64": np.float64, "df64": np.float64}
 
 
+# The raw handle of a device's current stream, without building a Stream
+# object: that took 2.9 us of the 15.8 us a call of Plan.solve spent on the
+# host, more than a pass of a small solve takes on the device.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream_handle(stream):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return stream.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 class Plan:
@@ -32,6 +40,7 @@ class Plan:
         self.h = tuple(float(v) for v in h)
         self.dtype = dtype
         self.torch_dtype = _TORCH[dtype]
+        self._shape = torch.Size(self.shape)
         self.handle = native.ipf_plan_create(self.n, self.h, dtype, flags, verbosity, _stream_handle(stream))
 
     @property
@@ -51,7 +60,7 @@ class Plan:
         return native.ipf_plan_spectrum_bytes(self.handle)
 
     def _check(self, t):
-        if not (t.is_cuda and t.dtype == self.torch_dtype and t.is_contiguous() and tuple(t.shape) == self.shape):
+        if not (t.is_cuda and t.dtype == self.torch_dtype and t.is_contiguous() and t.shape == self._shape):
             raise ValueError("expected a contiguous CUDA %s tensor of shape %s" % (self.torch_dtype, self.shape))
 
     def solve(self, src, out=None, stream=None):
