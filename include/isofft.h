@@ -116,8 +116,10 @@ enum {
  *   out        receives the plan handle (NULL on failure).
  *   n          {Nx, Ny, Nz}, each >= 1 and at most 1152: the doubled mesh
  *              (2N rounded up to one of 32, 48, 64, 96, 128, 192, 256, 384,
- *              512, 768, 1024, 1536, 2304) must fit the largest supported
- *              length, else IPF_UNSUPPORTED_SIZE.  1152^3 cells in FP32 need
+ *              512, 768, 1024, 1536, 2304 or, where the axis and dtype have
+ *              a faster pass of that length, 144, 288, 324, 432, 576, 648,
+ *              1152, 1296, 2048) must fit the largest supported length, else
+ *              IPF_UNSUPPORTED_SIZE; ipf_plan_padded_shape tells it.  1152^3 cells in FP32 need
  *              about 37 GB of device memory: a 24.5 GB workspace and a 6 GB
  *              spectrum, plus 24.5 GB of FP64 scratch while the spectrum is
  *              built.

@@ -38,10 +38,12 @@ def _spectrum_code():
 def _units():
     units = [("api", "api.cu", ["-DISOFFT_SPECTRUM_CODE=%s" % _spectrum_code()]), ("greens", "greens.cu", []),
              ("noalloc", "noalloc.cu", []), ("batch", "batch.cu", [])]
-    for real, tag in (("float", "f32"), ("double", "f64"), ("isofft::df64", "df64")):
-        for group, gname in ((1, "x"), (2, "y"), (3, "z")):
-            units.append(("passes_%s_%s" % (gname, tag), "passes_inst.cu",
-                          ["-DISOFFT_REAL=%s" % real, "-DISOFFT_GROUP=%d" % group]))
+    for real, tag, num in (("isofft::df64", "df64", 3), ("float", "f32", 1), ("double", "f64", 2)):
+        for group, gname in ((2, "y"), (3, "z"), (1, "x")):
+            for part in (1, 2):
+                units.append(("passes_%s%d_%s" % (gname, part, tag), "passes_inst.cu",
+                              ["-DISOFFT_REAL=%s" % real, "-DISOFFT_TYPE=%d" % num, "-DISOFFT_GROUP=%d" % group,
+                               "-DISOFFT_PART=%d" % part]))
     return units
 
 

@@ -182,11 +182,16 @@ int plan_zsh(int64_t Mz, int64_t Nz)
     return Mz == 2304 && Nz % (1 << kZBlockShift) == 0 ? kZBlockShift : 0;
 }
 
-int64_t choose_mesh(int64_t n)
+// The doubled mesh of a solve (false: an axis beyond the longest length).
+bool choose_mesh(const int64_t n[3], int dtype, int64_t M[3])
 {
-    for (int m : kSupportedM)
-        if (m >= 2 * n) return m;
-    return -1;
+    static_assert(kDtF32 == IPF_F32 && kDtF64 == IPF_F64 && kDtDf64 == IPF_DF64, "dtype numbering");
+    for (int a = 0; a < 3; ++a) {
+        M[a] = mesh_length(n[a], dtype, a);
+        if (M[a] < 0) return false;
+    }
+    if (plan_zsh(M[2], n[2])) M[1] = mesh_length(n[1], dtype, 1, true);
+    return true;
 }
 
 // bytes of one real of the source / potential arrays (FP64 for df64 solves);
@@ -201,9 +206,8 @@ int validate(const int64_t n[3], const double h[3], int dtype)
         if (n[a] < 1) return IPF_INVALID_ARG;
         if (!(h[a] > 0.0) || !isfinite(h[a])) return IPF_INVALID_ARG;
     }
-    for (int a = 0; a < 3; ++a)
-        if (choose_mesh(n[a]) < 0) return IPF_UNSUPPORTED_SIZE;
-    return IPF_OK;
+    int64_t M[3];
+    return choose_mesh(n, dtype, M) ? IPF_OK : IPF_UNSUPPORTED_SIZE;
 }
 
 // Widths divided by their minimum, rounded to a multiple of 2^-44 so that
@@ -867,9 +871,9 @@ int ipf_plan_create(ipf_plan_t *out, const int64_t n[3], const double h[3], int 
     if (!p) return IPF_OUT_OF_MEMORY;
     for (int a = 0; a < 3; ++a) {
         p->N[a] = n[a];
-        p->M[a] = choose_mesh(n[a]);
         p->h[a] = h[a];
     }
+    choose_mesh(n, dtype, p->M);  // validated above
     p->dtype = dtype;
     p->flags = flags;
     p->verbosity = verbosity;
@@ -972,7 +976,7 @@ int ipf_estimate_bytes(const int64_t n[3], const double h[3], int dtype, size_t 
     int rc = validate(n, h, dtype);
     if (rc) return rc;
     int64_t M[3];
-    for (int a = 0; a < 3; ++a) M[a] = choose_mesh(n[a]);
+    choose_mesh(n, dtype, M);
     size_t w = 2 * elem_size(dtype) * (size_t)n[2] * (size_t)M[1] * (size_t)(M[0] / 2);
     SpecKey key;
     double hmin;

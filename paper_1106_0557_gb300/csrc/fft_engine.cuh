@@ -139,11 +139,52 @@ ISOFFT_HD Cx<T> mul_root96(Cx<T> a)
     }
 }
 
+// cos(2 pi j / 36) over the first quadrant, for the radices 9, 18 and 36 (the
+// values to 40 digits, rounded).
+__host__ __device__ constexpr double cos36_base(int j)
+{
+    constexpr double b[10] = {1.0, 0.984807753012208, 0.9396926207859084, 0.8660254037844386, 0.766044443118978,
+                              0.6427876096865394, 0.5, 0.3420201433256687, 0.17364817766693036, 0.0};
+    return b[j];
+}
+__host__ __device__ constexpr double cos36(int j)
+{
+    j %= 36;
+    if (j < 0) j += 36;
+    if (j > 18) j = 36 - j;
+    return j > 9 ? -cos36_base(18 - j) : cos36_base(j);
+}
+
+// Multiply by W_R^e for R a divisor of 36 (as mul_root96).
+template <typename T, int R, int e>
+ISOFFT_HD Cx<T> mul_root36(Cx<T> a)
+{
+    constexpr int ee = ((e % R) + R) % R;
+    constexpr int j = ee * (36 / R);  // angle in units of 2 pi / 36
+    if constexpr (j != 0 && j % 9 != 0) a = crenorm(a);  // a product follows
+    if constexpr (j == 0) {
+        return a;
+    } else if constexpr (j == 9) {
+        return cmul_mi(a);  // -i
+    } else if constexpr (j == 18) {
+        return {-a.x, -a.y};
+    } else if constexpr (j == 27) {
+        return {-a.y, a.x};  // +i
+    } else {
+        constexpr T c = (T)cos36(j);
+        constexpr T s = (T)cos36(9 - j);
+        return {radd(rmul(a.x, c), rmul(a.y, s)), rsub(rmul(a.y, c), rmul(a.x, s))};
+    }
+}
+
 template <typename T, int R, int e>
 ISOFFT_HD Cx<T> mul_root(Cx<T> a)
 {
-    if constexpr (48 % R != 0) {
+    if constexpr (48 % R != 0 && 96 % R == 0) {
         return mul_root96<T, R, e>(a);
+    } else if constexpr (48 % R != 0) {
+        static_assert(36 % R == 0, "roots of unity of 96ths or 36ths");
+        return mul_root36<T, R, e>(a);
     } else {
         constexpr int ee = ((e % R) + R) % R;
         constexpr int j = ee * (48 / R);  // angle in units of 2 pi / 48
@@ -196,6 +237,25 @@ struct Dft<T, 3> {
         Cx<T> dif = crenorm(csub(a[1], a[2]));
         Cx<T> t = {a[0].x - (T)0.5 * sum.x, a[0].y - (T)0.5 * sum.y};
         Cx<T> u = {dif.y * s3, -dif.x * s3};  // -i s3 (a1 - a2)
+        a[0] = cadd(a[0], sum);
+        a[1] = cadd(t, u);
+        a[2] = csub(t, u);
+    }
+};
+
+// Float pairs: the sums of the radix 3 stay lazy like the other radices',
+// halving is exact, and the products only enter sums (142 -> 114 FP32
+// operations, against 128 of a radix 4).
+template <>
+struct Dft<df64, 3> {
+    static ISOFFT_HD void run(Cx<df64> (&a)[3])
+    {
+        constexpr df64 s3 = (df64)0.8660254037844387;  // sin(2 pi / 3)
+        const Cx<df64> sum = cadd(a[1], a[2]);
+        const Cx<df64> dif = crenorm(csub(a[1], a[2]));  // enters the products
+        const Cx<df64> h = {{-0.5f * sum.x.hi, -0.5f * sum.x.lo}, {-0.5f * sum.y.hi, -0.5f * sum.y.lo}};
+        const Cx<df64> t = cadd(a[0], h);
+        const Cx<df64> u = {rmul(dif.y, s3), -rmul(dif.x, s3)};  // -i s3 (a1 - a2)
         a[0] = cadd(a[0], sum);
         a[1] = cadd(t, u);
         a[2] = csub(t, u);
@@ -332,6 +392,18 @@ struct Dft<T, 32> {
 template <typename T>
 struct Dft<T, 24> {
     static ISOFFT_HD void run(Cx<T> (&a)[24]) { DftCT<T, 8, 3>::run(a); }
+};
+template <typename T>
+struct Dft<T, 9> {
+    static ISOFFT_HD void run(Cx<T> (&a)[9]) { DftCT<T, 3, 3>::run(a); }
+};
+template <typename T>
+struct Dft<T, 18> {
+    static ISOFFT_HD void run(Cx<T> (&a)[18]) { DftCT<T, 6, 3>::run(a); }
+};
+template <typename T>
+struct Dft<T, 36> {
+    static ISOFFT_HD void run(Cx<T> (&a)[36]) { DftCT<T, 12, 3>::run(a); }
 };
 template <typename T>
 struct Dft<T, 48> {
@@ -580,6 +652,17 @@ ISOFFT_SHAPE(Shape32, 1152, 12, 12, 12, 4, 2)
 ISOFFT_SHAPE(Shape32, 1536, 12, 12, 4, 4, 4, 2)
 ISOFFT_SHAPE(Shape32, 2304, 12, 12, 12, 4, 4)
 ISOFFT_SHAPE(Shape64, 1024, 8, 8, 8, 8, 2)
+// the lengths between: 9/8, 81/64 and 27/16 of a power of two
+ISOFFT_SHAPE(Shape32, 72, 12, 12, 6)
+ISOFFT_SHAPE(Shape32, 144, 12, 12, 12)
+ISOFFT_SHAPE(Shape32, 162, 18, 18, 9)
+ISOFFT_SHAPE(Shape32, 288, 12, 12, 12, 2)
+ISOFFT_SHAPE(Shape32, 324, 18, 18, 18)
+ISOFFT_SHAPE(Shape32, 432, 12, 12, 12, 3)
+ISOFFT_SHAPE(Shape32, 576, 12, 12, 12, 4)
+ISOFFT_SHAPE(Shape32, 648, 18, 18, 18, 2)
+ISOFFT_SHAPE(Shape32, 1296, 18, 18, 6, 6, 2)
+ISOFFT_SHAPE(Shape32, 2048, 8, 8, 8, 8, 4)
 #undef ISOFFT_SHAPE
 
 template <typename T, int L>
@@ -644,6 +727,25 @@ struct YShape<float, 768> {
     using Rad = Radices<24, 8, 4>;
 };
 
+#define ISOFFT_SHAPE_F32(S, L_, E_, ...)                  \
+    template <>                                           \
+    struct S<float, L_> {                                 \
+        static constexpr int E = E_;                      \
+        using Rad = Radices<__VA_ARGS__>;                 \
+    };
+// the lengths between (K2 + K4, us, at 256 x M/2 x 128 cells, and at the next
+// longer length of before): 288 20 + 20 (384: 33 + 33), 324 33 + 27, 432
+// 37 + 37 (512: 42 + 39), 576 46 + 41 (768: 72 + 66), 648 65 + 72, 1152
+// 91 + 112 (1536: 173 + 162), 1296 131 + 149, 2048 252 + 237 (2304: 197 + 261,
+// for 11 % fewer z lines)
+ISOFFT_SHAPE_F32(YShape, 288, 24, 24, 12)
+ISOFFT_SHAPE_F32(YShape, 432, 36, 36, 12)
+ISOFFT_SHAPE_F32(YShape, 576, 24, 24, 24)
+ISOFFT_SHAPE_F32(YShape, 648, 36, 36, 18)
+ISOFFT_SHAPE_F32(YShape, 1152, 48, 48, 24)
+ISOFFT_SHAPE_F32(YShape, 1296, 36, 36, 36)
+ISOFFT_SHAPE_F32(YShape, 2048, 32, 32, 32, 2)
+
 // The z pass holds two lines groups per tile and stages its prefetches in
 // shared memory.  512-point FP32 lines run 32 points per thread in two
 // stages (16 32): one exchange per transform instead of two with 8 8 8 (16
@@ -668,7 +770,8 @@ struct ZShape<float, 512> {
 // Measured, z pass alone: 128 points (16 8) 22.1 -> 20.4 us at 128^2 x 64;
 // 192 (24 8) 32.7 -> 26.7 us at 128^2 x 96; 256 (16 16) 38.9 -> 32.7 us at
 // 128^3; 384 (24 4 4) and 768 (24 8 4) 14-16 % (384^3: 1.124 -> 0.960 ms);
-// 1024 (32 32) 2.90 -> 2.79 ms at 512^3.
+// 1024 (32 32) 2.90 -> 2.79 ms at 512^3; 1536 (8 8 24 for 12 4 4 4 2)
+// 684 -> 577 us at 256 x 128 x 768.
 template <>
 struct ZShape<float, 128> {
     static constexpr int E = 16;
@@ -705,6 +808,26 @@ struct ZShape<float, 768> {
     using Rad = Radices<24, 8, 4>;
     static constexpr bool TW_REGS = true;
 };
+#define ISOFFT_ZSHAPE_F32(L_, E_, ...)                    \
+    template <>                                           \
+    struct ZShape<float, L_> {                            \
+        static constexpr int E = E_;                      \
+        using Rad = Radices<__VA_ARGS__>;                 \
+        static constexpr bool TW_REGS = true;             \
+    };
+// The lengths between take the radix order that leaves a thread the fewest
+// twiddles (a stage's twiddles are shared by the thread's butterflies where
+// the thread count is a multiple of the stage's stride): 56 us at 288 against
+// 90 at the next longer length of before (384), 107 against 198 at 576 (768),
+// 298 against 577 at 1152 (1536), 841 against 949 at 2048 (2304), on
+// 256 x 128 x M/2 cells.
+ISOFFT_ZSHAPE_F32(288, 24, 12, 24)
+ISOFFT_ZSHAPE_F32(324, 18, 18, 18)
+ISOFFT_ZSHAPE_F32(576, 24, 24, 24)
+ISOFFT_ZSHAPE_F32(1152, 24, 12, 4, 24)
+ISOFFT_ZSHAPE_F32(1536, 24, 8, 8, 24)
+ISOFFT_ZSHAPE_F32(2048, 32, 4, 16, 32)
+#undef ISOFFT_ZSHAPE_F32
 // 16-byte points on 768-point lines (one-column tiles of 128 threads): the
 // radix 12 goes last, where a thread's stage twiddles are shared by all its
 // butterflies (the thread count is a multiple of every stage's stride): 17
@@ -720,7 +843,8 @@ template <>
 struct ZShape<double, 768> : ZShape16B768 {};
 template <>
 struct ZShape<df64, 768> : ZShape16B768 {};
-// 2304-point lines read their twiddles from the table (a thread's share
+// 2304-point lines (and FP32 lines of 1296 points, at 36 points a thread: 469
+// us against 577 at 1536) read their twiddles from the table (a thread's share
 // would not fit in registers next to its points).  FP32 takes 24 points per
 // thread and three stages, so that a tile of two columns (16 bytes, the
 // narrowest tensor-copy row) fits 384 threads; 16-byte FP64-class points
@@ -729,6 +853,12 @@ struct ZShape<df64, 768> : ZShape16B768 {};
 // warps per SM.)
 template <typename T>
 struct ZShape<T, 2304> : Shape<T, 2304> {
+    static constexpr bool TW_REGS = false;
+};
+template <>
+struct ZShape<float, 1296> {
+    static constexpr int E = 36;
+    using Rad = Radices<36, 36>;
     static constexpr bool TW_REGS = false;
 };
 template <>
@@ -749,6 +879,16 @@ struct XShape<float, 256> {
     static constexpr int E = 16;
     using Rad = Radices<16, 16>;
 };
+// The lengths between, K1 + K5 in us at M/2 x 200 x 128 cells (M = 2 L) and at
+// the next longer length of before: 144 20 + 21 (192: 22 + 24), 288 33 + 37
+// (384: 39 + 43), 576 53 + 65 (768: 75 + 90), 1024 93 + 102 (1152: 123 + 143);
+// 162, 324 and 648 (25 + 27, 39 + 45, 98 + 104) cost about as much as 192, 384
+// and 768 do and save the other passes 16 % of their columns.
+ISOFFT_SHAPE_F32(XShape, 288, 24, 24, 12)
+ISOFFT_SHAPE_F32(XShape, 576, 24, 24, 24)
+ISOFFT_SHAPE_F32(XShape, 648, 36, 36, 18)
+ISOFFT_SHAPE_F32(XShape, 1024, 32, 32, 32)
+#undef ISOFFT_SHAPE_F32
 // K1's rows: FP32 rows of 768 and 1152 points run 24 points per thread in
 // three stages (two exchanges instead of three); measured 42 % and 22 %
 // faster than 12 points per thread, while K5 on the same rows was slower

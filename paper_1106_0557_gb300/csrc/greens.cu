@@ -89,7 +89,8 @@ k_cos_lines(double *__restrict__ oct, const Cx<double> *__restrict__ tw, int64_t
 }
 
 #define ISOFFT_DCT_LENGTHS(X) \
-    X(32) X(48) X(64) X(96) X(128) X(192) X(256) X(384) X(512) X(768) X(1024) X(1536) X(2304)
+    X(32) X(48) X(64) X(96) X(128) X(144) X(192) X(256) X(288) X(324) X(384) X(432) X(512) X(576) X(648) X(768) \
+    X(1024) X(1152) X(1296) X(1536) X(2048) X(2304)
 
 template <int L>
 static cudaError_t run_cos_lines(double *oct, const Cx<double> *tw, int64_t A, int64_t Cc, cudaStream_t st)
@@ -180,28 +181,27 @@ template size_t spectrum_elems<df64>(const int64_t *);
 void host_roots(int64_t n, int64_t count, double *re, double *im)
 {
     // e^{-2 pi i k/n}: reduce k to [0, n/8] by the exact symmetries of the
-    // circle (n is a multiple of 8 for every length used here; other n fall
+    // circle (n is a multiple of 4 for every length used here; other n fall
     // back to the direct angle).
     for (int64_t k = 0; k < count; ++k) {
         int64_t r = ((k % n) + n) % n;
         double c, s;  // cos and sin of 2 pi r / n
-        if (n % 8 == 0) {
-            const int64_t q = n / 8;
+        if (n % 4 == 0) {
             bool neg_s = false;
-            if (r > 4 * q) {  // lower half: sin negative
+            if (2 * r > n) {  // lower half: sin negative
                 r = n - r;
                 neg_s = true;
             }
             // r in [0, n/2]
             bool neg_c = false;
-            if (r > 2 * q) {  // second quadrant: cos(pi - a) = -cos a, sin same
-                r = 4 * q - r;
+            if (4 * r > n) {  // second quadrant: cos(pi - a) = -cos a, sin same
+                r = n / 2 - r;
                 neg_c = true;
             }
             // r in [0, n/4]
             double cc, ss;
-            if (r > q) {  // (q, 2q]: swap cos and sin of the complement
-                const double a = 2.0 * M_PI * (double)(2 * q - r) / (double)n;
+            if (8 * r > n) {  // past n/8: swap cos and sin of the complement
+                const double a = 2.0 * M_PI * (double)(n / 4 - r) / (double)n;
                 cc = sin(a);
                 ss = cos(a);
             } else {

@@ -9,10 +9,48 @@
 
 namespace isofft {
 
-// Doubled-mesh lengths the kernels are instantiated for (any M >= 2N - 1
-// gives the same cropped result, so a plan rounds 2N up to the next one).
-constexpr int kSupportedM[] = {32, 48, 64, 96, 128, 192, 256, 384, 512, 768, 1024, 1536, 2304};
+// Doubled-mesh lengths.  Any M >= 2N - 1 gives the same cropped result, so a
+// plan rounds 2N up, on each axis, to the next length that is worth taking
+// there for its dtype.  Powers of two and 3/2 of them (and 2304) serve every
+// axis; the lengths between are 9/8, 81/64 and 27/16 of a power of two, which
+// the kernels reach in two or three stages of 12 to 48 points a thread.  A
+// length that does not beat the next longer one on its axis is left out
+// there (times of one pass, us, of 256 x 200 x 128-cell meshes with the axis
+// at M/2 cells, half that for the 16-byte types):
+//   FP32 z:  288 56, 324 84, 384 90, 432 120, 512 99, 576 107, 648 226,
+//            768 199, 1024 230, 1152 298, 1296 469, 1536 577, 2048 841,
+//            2304 949: 432 and 648 are left out (y takes them: 37 against
+//            42 at 512, 65 + 72 against 72 + 66 at 768, with 16 % fewer z
+//            lines);
+//   FP32 x:  432 31 + 33 against 22 + 23 at 512: left out; elsewhere a few
+//            per cent on the x passes buy 9 to 16 % fewer columns;
+//   df64 z:  lines of powers of two hold more warps and no radix 3: 144 69
+//            (as 192), 288 126, 384 194, 512 154, 576 289, 768 401, 1024 347,
+//            1152 474, 1536 861, 2048 919, 2304 1316, so 144, 384 and 768 are
+//            not taken on z; 324 319, 432 226 and 648 658 on no axis;
+//   FP64 z:  144 220, 192 303, 288 509, 324 742, 384 673, 576 1112, 648 1550,
+//            768 1457, 1152 2455, 1296 3375, 1536 3373, 2048 4284, 2304 5416.
+enum { kDtF32 = 0, kDtF64 = 1, kDtDf64 = 2 };  // = ipf_dtype
+struct MeshLength {
+    int m;
+    unsigned char axes[3];  // by dtype: bit a set where axis a (x, y, z) takes it
+};
+constexpr MeshLength kMeshLengths[] = {
+    {32, {7, 7, 7}},   {48, {7, 7, 7}},   {64, {7, 7, 7}},   {96, {7, 7, 7}},   {128, {7, 7, 7}},  {144, {0, 7, 3}},
+    {192, {7, 7, 7}},  {256, {7, 7, 7}},  {288, {7, 7, 7}},  {324, {7, 0, 0}},  {384, {7, 7, 3}},  {432, {2, 0, 0}},
+    {512, {7, 7, 7}},  {576, {7, 7, 7}},  {648, {3, 0, 0}},  {768, {7, 7, 3}},  {1024, {7, 7, 7}}, {1152, {7, 7, 7}},
+    {1296, {7, 0, 0}}, {1536, {7, 7, 7}}, {2048, {7, 7, 7}}, {2304, {7, 7, 7}}};
 constexpr int kMaxM = 2304;
+// The doubled length of n cells on an axis (-1 beyond the longest).  `blocked`:
+// only the lengths whose y passes also run on a z-blocked workspace.
+inline int mesh_length(int64_t n, int dtype, int axis, bool blocked = false)
+{
+    for (const MeshLength &c : kMeshLengths) {
+        const bool basic = (c.m & (c.m - 1)) == 0 ? c.m != 2048 : (c.m % 9 != 0 || c.m == 2304);
+        if (c.m >= 2 * n && (c.axes[dtype] >> axis & 1) && (basic || !blocked)) return c.m;
+    }
+    return -1;
+}
 
 // Counts every kernel launch the library makes (ipf_launch_count).
 void count_launch();
@@ -68,6 +106,26 @@ cudaError_t launch_z_convolve(int L, void *W, const void *tw, const T *G, const 
 // Green's spectrum is stored in tiles of this width (0: unsupported L).
 template <typename T>
 int z_tile_for(int L);
+
+// The lengths between powers of two and 3/2 of them (passes_inst.cu, part
+// 2); the launchers above call these for lengths of their own that they lack.
+template <typename T>
+cudaError_t launch_x_forward_more(int L, const typename IoReal<T>::type *src, void *W, const void *tw, const void *rtw,
+                                  int Nx, int Ny, int My, int64_t nrows, int zsh, cudaStream_t st);
+template <typename T>
+cudaError_t launch_x_inverse_more(int L, const void *W, typename IoReal<T>::type *phi, const void *tw, const void *rtw,
+                                  int Nx, int Ny, int My, int64_t nrows, int zsh, cudaStream_t st);
+template <typename T>
+cudaError_t launch_y_forward_more(int L, void *W, const void *tw, int Ny, int Kx, int Nz, int zsh, unsigned *status,
+                                  int variant, cudaStream_t st);
+template <typename T>
+cudaError_t launch_y_inverse_more(int L, void *W, const void *tw, int Ny, int Kx, int Nz, int zsh, unsigned *status,
+                                  int variant, cudaStream_t st);
+template <typename T>
+cudaError_t launch_z_convolve_more(int L, void *W, const void *tw, const T *G, const T *Gs, T gscale, int Nz, int My,
+                                   int Kx, int zsh, unsigned *status, unsigned test_extra_tx, cudaStream_t st);
+template <typename T>
+int z_tile_for_more(int L);
 
 // Elements of one (k_y', kx tile) block of the cached spectrum: nkz x tx
 // values, padded so that every block starts on a 16-byte boundary (the z pass

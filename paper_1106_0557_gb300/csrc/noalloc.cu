@@ -40,13 +40,6 @@ namespace {
 std::mutex g_noalloc_mu;
 void *g_noalloc_ptr[64] = {};
 
-int64_t noalloc_mesh(int64_t n)
-{
-    for (int m : kSupportedM)
-        if (m >= 2 * n) return m;
-    return -1;
-}
-
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 // Host-side address of this device's copy of the array (set up on the first
@@ -169,7 +162,7 @@ extern "C" int ipf_solve_noalloc(const int64_t n[3], const double h[3], int dtyp
     double hmin = h[0];
     for (int a = 0; a < 3; ++a) {
         if (n[a] < 1 || !(h[a] > 0.0) || !isfinite(h[a])) return IPF_INVALID_ARG;
-        M[a] = noalloc_mesh(n[a]);
+        M[a] = mesh_length(n[a], dtype, a);
         if (M[a] < 0) return IPF_UNSUPPORTED_SIZE;
         if (h[a] < hmin) hmin = h[a];
     }

@@ -208,7 +208,8 @@ struct ColCfg {
     static constexpr int TX0 = 128 / (int)sizeof(Cx<T>);
     static constexpr int TXS = 32 / (int)sizeof(Cx<T>);  // one 32-byte sector
     static constexpr int pow2_floor(int v) { return v >= 2 ? 2 * pow2_floor(v / 2) : 1; }
-    static constexpr int TXT = TX0 * NT <= 512 ? TX0 : pow2_floor(512 / NT >= 1 ? 512 / NT : 1);
+    static constexpr int MAXT = E >= 40 ? 384 : 512;  // 40 or more points a thread: up to 168 registers
+    static constexpr int TXT = TX0 * NT <= MAXT ? TX0 : pow2_floor(MAXT / NT >= 1 ? MAXT / NT : 1);
     static constexpr int TXW = TXT >= TXS || TXS * NT > 1024 ? TXT : TXS;
     static constexpr int TX = NARROW ? (TXW > 1 ? TXW / 2 : 1) : TXW;
     static constexpr int THREADS = TX * NT;
@@ -237,13 +238,22 @@ constexpr size_t z_smem(int tx, int L, int rb)
 }
 constexpr int z_tile_width(int rb, int nt, int L, int e)
 {
-    // 16-byte points on 12-point lines of 384 and 768: tiles of 128 threads,
-    // three CTAs per SM (measured 23 % faster than one CTA of 256 threads at
-    // 255 registers, despite some spills under the 168-register cap)
+    // 16-byte points on 12-point lines of 384 to 768: tiles of 96 or 128
+    // threads, four or three CTAs per SM (at 384 and 768 measured 23 % faster
+    // than one CTA of 256 threads at 255 registers, despite some spills under
+    // the 168-register cap)
     if (rb == 8 && e == 12 && nt >= 32 && nt <= 64) return 64 / nt;
     int tx = rb == 4 ? 8 : 4;
-    while (tx > 1 && (2 * tx * nt > (e > 8 ? 512 : 1024) || z_smem(tx, L, rb) > 200 * 1024)) tx /= 2;
+    while (tx > 1 && (2 * tx * nt > (e > 8 ? 512 : 1024) || z_smem(tx, L, rb) > 208 * 1024)) tx /= 2;
     return tx;
+}
+// CTAs per SM the registers are capped for: two where a small CTA leaves room
+// (FP32 288-point lines: 192 threads of 168 registers twice, two exchange
+// buffers each).
+constexpr int z_min_blocks(int rb, int nt, int L, int e, int tx)
+{
+    if (rb == 8 && e == 12 && nt >= 32 && nt <= 64) return 384 / (2 * tx * nt);
+    return 2 * tx * nt <= 192 && 2 * (z_smem(tx, L, rb) + 1024) <= 228 * 1024 ? 2 : 1;
 }
 
 // SH: the line's shape (points per thread, radices, where the twiddles
@@ -260,36 +270,37 @@ struct ZCfg {
     // row of both line groups, whose staging regions lie a multiple of 128
     // bytes apart, so both land on the same half of the banks (a 2-way
     // conflict on every input read).  Line group 1 is therefore staged from
-    // plane -1 (zeros), one row later, which puts it on the other half.
-    static constexpr bool SHIFT = sizeof(T) == 4 && TX * (int)sizeof(Cx<T>) == 64;
-    static constexpr int ZROWS = LH + (SHIFT ? 1 : 0);  // rows staged per line group
-    // tensor boxes: NZB equal boxes of at most 256 planes per line group
-    // (exactly LH planes, or with SHIFT at least LH + 1 in boxes of an even
-    // number of rows, so that every box starts 128-byte aligned)
-    static constexpr int boxes()
+    // plane -1 (zeros), one row later, which puts it on the other half (with
+    // one tile per box, DBX below).
+    static constexpr bool SHIFT_FITS = sizeof(T) == 4 && TX * (int)sizeof(Cx<T>) == 64;
+    // tensor boxes: equal boxes of at most 256 planes per line group (exactly
+    // LH planes, or shifted at least LH + 1 in boxes of an even number of
+    // rows, so that every box starts 128-byte aligned)
+    static constexpr int boxes(bool shift)
     {
         int n = 1;
-        if (SHIFT) {
-            while ((ZROWS + n - 1) / n > 256) ++n;
+        if (shift) {
+            while ((LH + n) / n > 256) ++n;
         } else {
             while (LH % n != 0 || LH / n > 256) ++n;
         }
         return n;
     }
-    static constexpr int NZB = boxes();
-    static constexpr int BOXZ = SHIFT ? ((ZROWS + NZB - 1) / NZB + 1) / 2 * 2 : LH / NZB;
+    static constexpr int box_rows(bool shift)
+    {
+        const int n = boxes(shift);
+        return shift ? ((LH + n) / n + 1) / 2 * 2 : LH / n;
+    }
     static constexpr int EPC = (int)sizeof(Cx<T>) / 8;  // 8-byte tensor elements per complex
     static constexpr int GBLK = z_spec_block(TX, LH + 1, (int)sizeof(T));
     static constexpr size_t XCH = (size_t)L * COLS * sizeof(Cx<T>);
-    static constexpr size_t IN_GROUP = (size_t)NZB * BOXZ * TX * sizeof(Cx<T>);  // one line group
-    static constexpr size_t IN_SET = 2 * IN_GROUP;
     static constexpr size_t G_BLK = (size_t)GBLK * sizeof(T);
     static constexpr size_t G_SET = 2 * G_BLK;  // the blocks of k_y' = pr and of My/2 (pr = 0 only)
     // without register twiddles the CTA keeps the line's twiddle table in
     // shared memory (read by every stage, loaded once per CTA)
     static constexpr bool TWR = SH::TW_REGS;
     static constexpr size_t TWS = TWR ? 0 : (size_t)L * sizeof(Cx<T>);
-    static constexpr int MIN_BLOCKS = sizeof(T) == 8 && E == 12 && NT >= 32 && NT <= 64 ? 3 : 1;
+    static constexpr int MIN_BLOCKS = z_min_blocks((int)sizeof(T), NT, L, E, TX);
     // Two exchange buffers used in turn need one CTA barrier per exchange
     // instead of two; the input is then staged once per tile (the next
     // tile's copies start after the first exchange's barrier, when every
@@ -299,12 +310,17 @@ struct ZCfg {
     // input set twice as wide (k_z_convolve_pairs: 2304-point lines, and the
     // 768-point lines of 16-byte points, 6.93 -> 6.62 ms for a df64 384^3
     // solve's z pass).
-    static constexpr size_t SMEM_DBX = 2 * XCH + IN_SET + 2 * G_SET + 16 + TWS;
-    // 16-byte points on 1-column tiles copy 16-byte rows; two tiles per box
-    // (the paired form) make them 32 bytes
-    static constexpr bool PAIR_NARROW = sizeof(Cx<T>) == 16 && TX == 1;
+    static constexpr size_t SMEM_DBX =
+        2 * XCH + (size_t)2 * boxes(SHIFT_FITS) * box_rows(SHIFT_FITS) * TX * sizeof(Cx<T>) + 2 * G_SET + 16 + TWS;
+    // tiles with 16-byte copy rows (16-byte points on 1-column tiles, the
+    // longest FP32 lines): two tiles per box make them 32 bytes
+    static constexpr bool PAIR_NARROW = TX * sizeof(Cx<T>) == 16 && (sizeof(Cx<T>) == 16 || L > 1536);
     static constexpr bool DBX =
         !PAIR_NARROW && SMEM_DBX <= 227 * 1024 && MIN_BLOCKS * (SMEM_DBX + 1024) <= 228 * 1024;
+    static constexpr bool SHIFT = SHIFT_FITS && DBX;
+    static constexpr int NZB = boxes(SHIFT), BOXZ = box_rows(SHIFT);
+    static constexpr size_t IN_GROUP = (size_t)NZB * BOXZ * TX * sizeof(Cx<T>);  // one line group
+    static constexpr size_t IN_SET = 2 * IN_GROUP;
     static constexpr int NXB = DBX ? 2 : 1;  // exchange buffers
     static constexpr int NIN = DBX ? 1 : 2;  // input sets of one tile's width
     static constexpr size_t OFF_IN = NXB * XCH, OFF_G = OFF_IN + NIN * IN_SET, OFF_BAR = OFF_G + 2 * G_SET,
@@ -326,7 +342,7 @@ struct ZCfg {
     static_assert(MIN_BLOCKS * SMEM <= 227 * 1024, "z pass CTAs per SM exceed shared memory");
     static_assert(THREADS <= 1024, "z tile too large");
     static_assert(SMEM <= 227 * 1024, "z tile exceeds shared memory");
-    static_assert((SHIFT ? BOXZ * NZB >= ZROWS : BOXZ * NZB == LH) && BOXZ <= 256,
+    static_assert((SHIFT ? BOXZ * NZB > LH : BOXZ * NZB == LH) && BOXZ <= 256,
                   "tensor boxes must cover the half line");
     static_assert(TX * sizeof(Cx<T>) % 16 == 0, "tensor box rows must be multiples of 16 bytes");
     static_assert(XCH % 128 == 0 && IN_GROUP % 128 == 0 && ((size_t)BOXZ * TX * sizeof(Cx<T>)) % 128 == 0,

@@ -3,6 +3,9 @@
 //   -DISOFFT_REAL=float|double|isofft::df64   the arithmetic type
 //   -DISOFFT_GROUP=1|2|3         1: x passes (K1, K5), 2: y passes (K2, K4),
 //                                3: z pass (K3)
+//   -DISOFFT_PART=1|2            the line lengths of powers of two and 3/2 of
+//                                them (and 2304), or those between
+//   -DISOFFT_TYPE=1|2|3          the same type as a number: float, double, df64
 // so that the instantiations compile in parallel.
 #include <atomic>
 
@@ -14,6 +17,12 @@
 #endif
 #ifndef ISOFFT_GROUP
 #error "define ISOFFT_GROUP"
+#endif
+#ifndef ISOFFT_PART
+#error "define ISOFFT_PART"
+#endif
+#ifndef ISOFFT_TYPE
+#error "define ISOFFT_TYPE"
 #endif
 
 namespace isofft {
@@ -64,10 +73,40 @@ static cudaError_t launch_pass(void (*kernel)(K...), dim3 grid, int threads, siz
     return e;
 }
 
+// Row lengths (Mx / 2) and column lengths (My, Mz) of each part, for the axes
+// and dtypes that kMeshLengths (launch.h) names.
+#if ISOFFT_PART == 1
 #define ISOFFT_ROW_LENGTHS(X) \
     X(16) X(24) X(32) X(48) X(64) X(96) X(128) X(192) X(256) X(384) X(512) X(768) X(1152)
-#define ISOFFT_COL_LENGTHS(X) \
+#define ISOFFT_Y_LENGTHS(X) \
     X(32) X(48) X(64) X(96) X(128) X(192) X(256) X(384) X(512) X(768) X(1024) X(1536) X(2304)
+#if ISOFFT_TYPE == 3
+#define ISOFFT_Z_LENGTHS(X) X(32) X(48) X(64) X(96) X(128) X(192) X(256) X(512) X(1024) X(1536) X(2304)
+#else
+#define ISOFFT_Z_LENGTHS(X) ISOFFT_Y_LENGTHS(X)
+#endif
+#elif ISOFFT_TYPE == 1
+#define ISOFFT_ROW_LENGTHS(X) X(144) X(162) X(288) X(324) X(576) X(648) X(1024)
+#define ISOFFT_Y_LENGTHS(X) X(288) X(324) X(432) X(576) X(648) X(1152) X(1296) X(2048)
+#define ISOFFT_Z_LENGTHS(X) X(288) X(324) X(576) X(1152) X(1296) X(2048)
+#else
+#define ISOFFT_ROW_LENGTHS(X) X(72) X(144) X(288) X(576) X(1024)
+#define ISOFFT_Y_LENGTHS(X) X(144) X(288) X(576) X(1152) X(2048)
+#if ISOFFT_TYPE == 3
+#define ISOFFT_Z_LENGTHS(X) X(288) X(576) X(1152) X(2048)
+#else
+#define ISOFFT_Z_LENGTHS(X) ISOFFT_Y_LENGTHS(X)
+#endif
+#endif
+
+// Each launcher tries its part's lengths; part 1's falls through to part 2's.
+#if ISOFFT_PART == 1
+#define ISOFFT_LAUNCHER(name) name
+#define ISOFFT_OTHERWISE(call) return call
+#else
+#define ISOFFT_LAUNCHER(name) name##_more
+#define ISOFFT_OTHERWISE(call)
+#endif
 
 // Resident CTAs per SM of a kernel on the current device (queried once).
 template <typename F>
@@ -147,7 +186,7 @@ static cudaError_t run_x_inverse(const void *W, In<T> *phi, const void *tw, cons
 }
 
 template <typename R_>
-cudaError_t launch_x_forward(int L, const In<R_> *src, void *W, const void *tw, const void *rtw, int Nx,
+cudaError_t ISOFFT_LAUNCHER(launch_x_forward)(int L, const In<R_> *src, void *W, const void *tw, const void *rtw, int Nx,
                                  int Ny, int My, int64_t nrows, int zsh, cudaStream_t st)
 {
     switch (L) {
@@ -155,11 +194,13 @@ cudaError_t launch_x_forward(int L, const In<R_> *src, void *W, const void *tw, 
     case n: return run_x_forward<R_, n>(src, W, tw, rtw, Nx, Ny, My, nrows, zsh, st);
         ISOFFT_ROW_LENGTHS(X_)
 #undef X_
-    default: return cudaErrorInvalidValue;
+    default: break;
     }
+    ISOFFT_OTHERWISE(launch_x_forward_more<R_>(L, src, W, tw, rtw, Nx, Ny, My, nrows, zsh, st));
+    return cudaErrorInvalidValue;
 }
 template <typename R_>
-cudaError_t launch_x_inverse(int L, const void *W, In<R_> *phi, const void *tw, const void *rtw, int Nx,
+cudaError_t ISOFFT_LAUNCHER(launch_x_inverse)(int L, const void *W, In<R_> *phi, const void *tw, const void *rtw, int Nx,
                                  int Ny, int My, int64_t nrows, int zsh, cudaStream_t st)
 {
     switch (L) {
@@ -167,23 +208,27 @@ cudaError_t launch_x_inverse(int L, const void *W, In<R_> *phi, const void *tw, 
     case n: return run_x_inverse<R_, n>(W, phi, tw, rtw, Nx, Ny, My, nrows, zsh, st);
         ISOFFT_ROW_LENGTHS(X_)
 #undef X_
-    default: return cudaErrorInvalidValue;
+    default: break;
     }
+    ISOFFT_OTHERWISE(launch_x_inverse_more<R_>(L, W, phi, tw, rtw, Nx, Ny, My, nrows, zsh, st));
+    return cudaErrorInvalidValue;
 }
-template cudaError_t launch_x_forward<Real>(int, const In<Real> *, void *, const void *, const void *, int, int,
+template cudaError_t ISOFFT_LAUNCHER(launch_x_forward)<Real>(int, const In<Real> *, void *, const void *, const void *, int, int,
                                             int, int64_t, int, cudaStream_t);
-template cudaError_t launch_x_inverse<Real>(int, const void *, In<Real> *, const void *, const void *, int, int,
+template cudaError_t ISOFFT_LAUNCHER(launch_x_inverse)<Real>(int, const void *, In<Real> *, const void *, const void *, int, int,
                                             int, int64_t, int, cudaStream_t);
 #endif
 
 #if ISOFFT_GROUP == 2
+constexpr bool kBlocked = ISOFFT_PART == 1;  // mesh_length's `blocked` lengths
 template <typename T, int L, bool FWD, bool NARROW>
 static cudaError_t run_y_tile(void *W, const void *tw, int Ny, int Kx, int Nz, int zsh, cudaStream_t st)
 {
     using C = ColCfg<T, L, NARROW>;
     static std::atomic<uint64_t> done0{0}, doneb{0};
     // plain and z-blocked workspace instances
-    auto *k = zsh ? (FWD ? k_y_forward<T, L, NARROW, true> : k_y_inverse<T, L, NARROW, true>)
+    if (zsh && !kBlocked) return cudaErrorInvalidValue;
+    auto *k = zsh ? (FWD ? k_y_forward<T, L, NARROW, kBlocked> : k_y_inverse<T, L, NARROW, kBlocked>)
                   : (FWD ? k_y_forward<T, L, NARROW, false> : k_y_inverse<T, L, NARROW, false>);
     if (!w_blocks_ok(Nz, zsh)) return cudaErrorInvalidValue;
     cudaError_t e = ensure_smem(k, C::SMEM, zsh ? doneb : done0);
@@ -201,7 +246,8 @@ static cudaError_t run_y_stream(void *W, const void *tw, int Ny, int Kx, int Nz,
     static std::atomic<int> slots0{0}, slotsb{0};
     if ((uintptr_t)W & 15) return cudaErrorMisalignedAddress;
     // plain and z-blocked workspace instances
-    auto *k = zsh ? k_y_pass<T, L, FWD, true> : k_y_pass<T, L, FWD, false>;
+    if (zsh && !kBlocked) return cudaErrorInvalidValue;
+    auto *k = zsh ? k_y_pass<T, L, FWD, kBlocked> : k_y_pass<T, L, FWD, false>;
     cudaError_t e = ensure_smem(k, SMEM, zsh ? doneb : done0);
     if (e != cudaSuccess) return e;
     const int ntx = (Kx + C::TX - 1) / C::TX;
@@ -251,32 +297,36 @@ static cudaError_t run_y(void *W, const void *tw, int Ny, int Kx, int Nz, int zs
     return run_y_tile<T, L, FWD, false>(W, tw, Ny, Kx, Nz, zsh, st);
 }
 template <typename R_>
-cudaError_t launch_y_forward(int L, void *W, const void *tw, int Ny, int Kx, int Nz, int zsh, unsigned *status,
+cudaError_t ISOFFT_LAUNCHER(launch_y_forward)(int L, void *W, const void *tw, int Ny, int Kx, int Nz, int zsh, unsigned *status,
                              int variant, cudaStream_t st)
 {
     switch (L) {
 #define X_(n) \
     case n: return run_y<R_, n, true>(W, tw, Ny, Kx, Nz, zsh, status, variant, st);
-        ISOFFT_COL_LENGTHS(X_)
+        ISOFFT_Y_LENGTHS(X_)
 #undef X_
-    default: return cudaErrorInvalidValue;
+    default: break;
     }
+    ISOFFT_OTHERWISE(launch_y_forward_more<R_>(L, W, tw, Ny, Kx, Nz, zsh, status, variant, st));
+    return cudaErrorInvalidValue;
 }
 template <typename R_>
-cudaError_t launch_y_inverse(int L, void *W, const void *tw, int Ny, int Kx, int Nz, int zsh, unsigned *status,
+cudaError_t ISOFFT_LAUNCHER(launch_y_inverse)(int L, void *W, const void *tw, int Ny, int Kx, int Nz, int zsh, unsigned *status,
                              int variant, cudaStream_t st)
 {
     switch (L) {
 #define X_(n) \
     case n: return run_y<R_, n, false>(W, tw, Ny, Kx, Nz, zsh, status, variant, st);
-        ISOFFT_COL_LENGTHS(X_)
+        ISOFFT_Y_LENGTHS(X_)
 #undef X_
-    default: return cudaErrorInvalidValue;
+    default: break;
     }
+    ISOFFT_OTHERWISE(launch_y_inverse_more<R_>(L, W, tw, Ny, Kx, Nz, zsh, status, variant, st));
+    return cudaErrorInvalidValue;
 }
-template cudaError_t launch_y_forward<Real>(int, void *, const void *, int, int, int, int, unsigned *, int,
+template cudaError_t ISOFFT_LAUNCHER(launch_y_forward)<Real>(int, void *, const void *, int, int, int, int, unsigned *, int,
                                             cudaStream_t);
-template cudaError_t launch_y_inverse<Real>(int, void *, const void *, int, int, int, int, unsigned *, int,
+template cudaError_t ISOFFT_LAUNCHER(launch_y_inverse)<Real>(int, void *, const void *, int, int, int, int, unsigned *, int,
                                             cudaStream_t);
 #endif
 
@@ -300,14 +350,14 @@ static cudaError_t run_z(void *W, const void *tw, const T *G, const T *Gs, T gsc
         if constexpr (C::DBX)
             return k_z_convolve<T, L>;
         else
-            return k_z_convolve_pairs<T, L, kZBlockShift>;
+            return k_z_convolve_pairs<T, L, L == 2304 ? kZBlockShift : 0>;
     }();
     static std::atomic<uint64_t> done0{0}, doneb{0};
     static std::atomic<int> slots0{0}, slotsb{0};
     if (((uintptr_t)W & 15) || ((uintptr_t)G & 15)) return cudaErrorMisalignedAddress;
     // the z-blocked workspace is read by the paired form only, in boxes of
     // whole blocks
-    if (!w_blocks_ok(Nz, zsh) || (zsh && (C::DBX || zsh != kZBlockShift || C::BOXZ % (1 << zsh))))
+    if (!w_blocks_ok(Nz, zsh) || (zsh && (L != 2304 || C::DBX || zsh != kZBlockShift || C::BOXZ % (1 << zsh))))
         return cudaErrorInvalidValue;
     const auto kernel = zsh ? kernelb : kernel0;
     cudaError_t e = ensure_smem(kernel, C::SMEM, zsh ? doneb : done0);
@@ -343,32 +393,36 @@ static cudaError_t run_z(void *W, const void *tw, const T *G, const T *Gs, T gsc
                        Nz, My, Kx, units, status, test_extra_tx);
 }
 template <typename R_>
-cudaError_t launch_z_convolve(int L, void *W, const void *tw, const R_ *G, const R_ *Gs, R_ gscale,
+cudaError_t ISOFFT_LAUNCHER(launch_z_convolve)(int L, void *W, const void *tw, const R_ *G, const R_ *Gs, R_ gscale,
                                   int Nz, int My, int Kx, int zsh, unsigned *status, unsigned test_extra_tx,
                                   cudaStream_t st)
 {
     switch (L) {
 #define X_(n) \
     case n: return run_z<R_, n>(W, tw, G, Gs, gscale, Nz, My, Kx, zsh, status, test_extra_tx, st);
-        ISOFFT_COL_LENGTHS(X_)
+        ISOFFT_Z_LENGTHS(X_)
 #undef X_
-    default: return cudaErrorInvalidValue;
+    default: break;
     }
+    ISOFFT_OTHERWISE(launch_z_convolve_more<R_>(L, W, tw, G, Gs, gscale, Nz, My, Kx, zsh, status, test_extra_tx, st));
+    return cudaErrorInvalidValue;
 }
 template <typename R_>
-int z_tile_for(int L)
+int ISOFFT_LAUNCHER(z_tile_for)(int L)
 {
     switch (L) {
 #define X_(n) \
     case n: return ZCfg<R_, n>::TX;
-        ISOFFT_COL_LENGTHS(X_)
+        ISOFFT_Z_LENGTHS(X_)
 #undef X_
-    default: return 0;
+    default: break;
     }
+    ISOFFT_OTHERWISE(z_tile_for_more<R_>(L));
+    return 0;
 }
-template cudaError_t launch_z_convolve<Real>(int, void *, const void *, const Real *, const Real *, Real, int,
+template cudaError_t ISOFFT_LAUNCHER(launch_z_convolve)<Real>(int, void *, const void *, const Real *, const Real *, Real, int,
                                              int, int, int, unsigned *, unsigned, cudaStream_t);
-template int z_tile_for<Real>(int);
+template int ISOFFT_LAUNCHER(z_tile_for)<Real>(int);
 #endif
 
 }  // namespace isofft
