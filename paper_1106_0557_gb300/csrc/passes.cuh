@@ -87,11 +87,9 @@ __device__ __forceinline__ void cp_async_wait()
 //   64-byte rows:        p ^ (bit 3 ^ bit 4 of p)
 //   32- and 16-byte rows: p ^ (bits 3-4 of p)
 // which makes every exchange pattern of the column shapes conflict-free or
-// nearly so (counted per pattern, per half- or quarter-warp).  The z pass
-// swizzles only the 32-byte rows of its 2304-point lines, where 42 % of its
-// shared wavefronts were conflict replays: on 64-byte rows the per-access
-// address arithmetic cost it more (measured at 768 points) than the
-// conflicts it removes, and the register-twiddle shapes would spill.
+// nearly so (counted per pattern, per half- or quarter-warp).  The z pass uses
+// them only on FP64-class 2304-point lines; its FP32 lines swizzle their
+// first exchange alone (ZXch).
 template <typename T, int L, int E, int COLS, bool SWIZZLE = true>
 struct ColXch {
     static constexpr int ROW_BYTES = COLS * (int)sizeof(Cx<T>);
@@ -236,6 +234,12 @@ constexpr size_t z_smem(int tx, int L, int rb)
            + 2 * 2 * (size_t)z_spec_block(tx, L / 2 + 1, rb) * rb  // spectrum blocks, two sets
            + 16;                                                      // mbarriers
 }
+// ... and with two exchange buffers and one input set (a bound)
+constexpr size_t z_smem_dbx(int tx, int L, int rb)
+{
+    return 2 * (size_t)L * 2 * tx * 2 * rb + (size_t)(L + 16) * tx * 2 * rb +
+           4 * (size_t)z_spec_block(tx, L / 2 + 1, rb) * rb + 16;
+}
 constexpr int z_tile_width(int rb, int nt, int L, int e)
 {
     // 16-byte points on 12-point lines of 384 to 768: tiles of 96 or 128
@@ -247,13 +251,20 @@ constexpr int z_tile_width(int rb, int nt, int L, int e)
     while (tx > 1 && (2 * tx * nt > (e > 8 ? 512 : 1024) || z_smem(tx, L, rb) > 208 * 1024)) tx /= 2;
     return tx;
 }
-// CTAs per SM the registers are capped for: two where a small CTA leaves room
-// (FP32 288-point lines: 192 threads of 168 registers twice, two exchange
-// buffers each).
+// CTAs per SM the registers are capped for.  FP32: enough for 16 warps of 128
+// registers (up to 16 points a thread) or 12 of 168 (up to 24), where their
+// shared memory fits too; without the cap the compiler takes 154 to 244 and
+// half the warps.  Nothing spills: z pass on 256 x 128 x L/2 cells, 96 points
+// 24.6 -> 23.2 us, 128 28.6 -> 24.4, 192 36.9 -> 34.6, 256 55.1 -> 47.2.
+// 16-byte points: two CTAs where a small one leaves room.
 constexpr int z_min_blocks(int rb, int nt, int L, int e, int tx)
 {
     if (rb == 8 && e == 12 && nt >= 32 && nt <= 64) return 384 / (2 * tx * nt);
-    return 2 * tx * nt <= 192 && 2 * (z_smem(tx, L, rb) + 1024) <= 228 * 1024 ? 2 : 1;
+    if (rb == 8) return 2 * tx * nt <= 192 && 2 * (z_smem(tx, L, rb) + 1024) <= 228 * 1024 ? 2 : 1;
+    const int threads = 2 * tx * nt, want = (e <= 16 ? 512 : 384) / threads;
+    const int fit = (int)((size_t)228 * 1024 / (z_smem_dbx(tx, L, rb) + 1024));
+    const int n = want < fit ? want : fit;
+    return e <= 24 && n > 1 ? n : 1;
 }
 
 // SH: the line's shape (points per thread, radices, where the twiddles
@@ -334,10 +345,10 @@ struct ZCfg {
                           ((size_t)BOXZ * PTX * sizeof(Cx<T>)) % 128 == 0),
                   "paired z tiles: layout and 128-byte aligned copy destinations");
     // rows of 32 bytes or less put several positions on one bank row: the
-    // lines that keep their twiddles in shared memory swizzle them (the
-    // register-twiddle shapes would spill under the extra address registers;
-    // wider rows go without, see ColXch)
-    static constexpr bool SWZ = !TWR && COLS * sizeof(Cx<T>) <= 32;
+    // FP64-class lines that keep their twiddles in shared memory swizzle them
+    // (the register-twiddle shapes would spill under the extra address
+    // registers); FP32 swizzles its first exchange in ZXch
+    static constexpr bool SWZ = sizeof(T) == 8 && !TWR && COLS * sizeof(Cx<T>) <= 32;
     static_assert(DBX || SMEM == z_smem(TX, L, (int)sizeof(T)) + TWS, "z pass shared-memory layout");
     static_assert(MIN_BLOCKS * SMEM <= 227 * 1024, "z pass CTAs per SM exceed shared memory");
     static_assert(THREADS <= 1024, "z tile too large");
@@ -786,20 +797,53 @@ struct ZXch {
     {
         using G = StageGeom<L, E, NS, R>;
         Cx<T> *s = buf(k);
+        // FP32 rows narrower than the banks hold P positions per bank row.  The
+        // first stage's writes of neighbouring threads lie R positions apart,
+        // all on one part of the banks (a P-way conflict); position p goes to
+        // row p ^ ((p >> S) & (P - 1)), S the power of two in R, which differs
+        // between neighbours and is, on the reading side, the same for all of a
+        // thread's points (or takes P values).  Later stages write neighbours
+        // to neighbouring rows.  z pass on 256 x 128 x L/2 cells: 768 points
+        // 198 -> 186 us, 1024 230 -> 216, 1152 298 -> 273, 1536 577 -> 478,
+        // 2048 841 -> 747, 2304 949 -> 874 (where every exchange was swizzled
+        // by ColXch's rule before).
+        constexpr int P = !SWZ && sizeof(T) == 4 && NS == 1 && COLS * sizeof(Cx<T>) < 128 ? 128 / (COLS * (int)sizeof(Cx<T>)) : 1;
+        constexpr int S = ctz(R);
+        if constexpr (P > 1) {
+            static_assert((1 << S) >= P && G::NT % (1 << S) == 0, "swizzle of the first exchange");
 #pragma unroll
-        for (int q = 0; q < G::B; ++q)
+            for (int q = 0; q < G::B; ++q) {
+                const int j = t + q * G::NT, u = (R >> S) * j;
+                Cx<T> *b = s + R * j * COLS + c;
 #pragma unroll
-            for (int r = 0; r < R; ++r) s[Rows::row(G::out_pos(t, q, r)) * COLS + c] = v[q + r * G::B];
+                for (int r = 0; r < R; ++r)
+                    b[((r & ~(P - 1)) + ((r & (P - 1)) ^ ((u + (r >> S)) & (P - 1)))) * COLS] = v[q + r * G::B];
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < G::B; ++q)
+#pragma unroll
+                for (int r = 0; r < R; ++r) s[Rows::row(G::out_pos(t, q, r)) * COLS + c] = v[q + r * G::B];
+        }
         if constexpr (PREWAIT) {
             if (threadIdx.x == 0) bulk_wait_read_all();
         }
         __syncthreads();
         hook(k);
+        if constexpr (P > 1) {
 #pragma unroll
-        for (int m = 0; m < E; ++m) v[m] = s[Rows::row(t + m * G::NT) * COLS + c];
+            for (int m = 0; m < E; ++m) {
+                constexpr int step = G::NT >> S;
+                v[m] = s[((t ^ (((t >> S) + m * step) & (P - 1))) + m * G::NT) * COLS + c];
+            }
+        } else {
+#pragma unroll
+            for (int m = 0; m < E; ++m) v[m] = s[Rows::row(t + m * G::NT) * COLS + c];
+        }
         if constexpr (!DB) __syncthreads();
         ++k;
     }
+    static constexpr int ctz(int n) { return n & 1 ? 0 : 1 + ctz(n / 2); }
 };
 
 
