@@ -175,12 +175,23 @@ struct ipf_plan_s {
 
 namespace {
 
-// z blocking of the workspace (w_row): on 2304-point z lines, blocks of
-// 2^kZBlockShift planes, where the plane count allows.
-int plan_zsh(int64_t Mz, int64_t Nz)
+// z blocking of the workspace (w_row): where the z pass copies rows of 32 or
+// 16 bytes (lines of 768 points and more), one row per plane, and the planes
+// are so large that each row lies in a memory page of its own (2 MB).  In
+// blocks of 16 planes the rows of a line come from 16 times fewer pages: K3
+// 2373 -> 1612 us at FP32 768 x 384 x 384 (planes of 4.7 MB), 2730 -> 1572 at
+// 512^3, 924 -> 813 at 384^3 (2.4 MB); at 309^3 (1.7 MB) 566 -> 590, and on
+// planes of 1 MB and less the solve is no faster (366 -> 369 us at
+// 256 x 128 x 384), so those stay plain.  2304-point lines of whole blocks
+// take them for every dtype and plane.
+int plan_zsh(const int64_t M[3], int64_t Nz, int dtype)
 {
-    return Mz == 2304 && Nz % (1 << kZBlockShift) == 0 ? kZBlockShift : 0;
+    if (M[2] == 2304 && Nz % (1 << kZBlockShift) == 0) return kZBlockShift;
+    const int64_t plane = M[1] * (M[0] / 2) * 8;
+    return dtype == IPF_F32 && z_blocks((int)M[2], true) && plane >= (2 << 20) ? kZBlockShift : 0;
 }
+// Planes of the workspace: whole blocks.
+int64_t w_planes(int64_t Nz, int zsh) { return ((Nz + (1 << zsh) - 1) >> zsh) << zsh; }
 
 // The doubled mesh of a solve (false: an axis beyond the longest length).
 bool choose_mesh(const int64_t n[3], int dtype, int64_t M[3])
@@ -190,7 +201,8 @@ bool choose_mesh(const int64_t n[3], int dtype, int64_t M[3])
         M[a] = mesh_length(n[a], dtype, a);
         if (M[a] < 0) return false;
     }
-    if (plan_zsh(M[2], n[2])) M[1] = mesh_length(n[1], dtype, 1, true);
+    // only FP32 has blocked y passes of every length
+    if (dtype != IPF_F32 && plan_zsh(M, n[2], dtype)) M[1] = mesh_length(n[1], dtype, 1, true);
     return true;
 }
 
@@ -893,9 +905,9 @@ int ipf_plan_create(ipf_plan_t *out, const int64_t n[3], const double h[3], int 
     p->key.device = p->device;
     p->key.dtype = dtype;
     for (int a = 0; a < 3; ++a) p->key.M[a] = p->M[a];
-    p->zsh = plan_zsh(p->M[2], p->N[2]);
+    p->zsh = plan_zsh(p->M, p->N[2], dtype);
 
-    p->W_bytes = 2 * elem_size(dtype) * (size_t)p->N[2] * (size_t)p->M[1] * (size_t)(p->M[0] / 2);
+    p->W_bytes = 2 * elem_size(dtype) * (size_t)w_planes(p->N[2], p->zsh) * (size_t)p->M[1] * (size_t)(p->M[0] / 2);
     ce = dev_alloc(&p->W, p->W_bytes, "workspace");
     if (ce != cudaSuccess) {
         rc = cuda_status(ce);
@@ -977,7 +989,8 @@ int ipf_estimate_bytes(const int64_t n[3], const double h[3], int dtype, size_t 
     if (rc) return rc;
     int64_t M[3];
     choose_mesh(n, dtype, M);
-    size_t w = 2 * elem_size(dtype) * (size_t)n[2] * (size_t)M[1] * (size_t)(M[0] / 2);
+    size_t w = 2 * elem_size(dtype) * (size_t)w_planes(n[2], plan_zsh(M, n[2], dtype)) * (size_t)M[1] *
+               (size_t)(M[0] / 2);
     SpecKey key;
     double hmin;
     normalized_widths(h, key.hn, &hmin);

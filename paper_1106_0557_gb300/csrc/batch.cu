@@ -258,7 +258,7 @@ __device__ __forceinline__ void batch_z_compute(const BatchGrid &g, uint32_t idx
     // every sub-group meets the packed column's barriers (the sub-groups'
     // tiles differ in xt)
     z_tile<float, L, TX, true, typename B::SH>(s_in + grp * (Lh + (C::SHIFT ? 1 : 0)) * TX, sg, pr, xt, g.W, g.Gs, g.gscale, g.Nz,
-                               g.My, Kx, 0, c, grp, t,
+                               g.My, Kx, c, grp, t,
                                twr, g.tw_z, xch, [] { return true; });
 }
 

@@ -41,6 +41,12 @@ constexpr MeshLength kMeshLengths[] = {
     {512, {7, 7, 7}},  {576, {7, 7, 7}},  {648, {3, 0, 0}},  {768, {7, 7, 3}},  {1024, {7, 7, 7}}, {1152, {7, 7, 7}},
     {1296, {7, 0, 0}}, {1536, {7, 7, 7}}, {2048, {7, 7, 7}}, {2304, {7, 7, 7}}};
 constexpr int kMaxM = 2304;
+// Whether z lines of length Mz have an instance on a z-blocked workspace.
+constexpr bool z_blocks(int Mz, bool f32)
+{
+    return Mz == 2304 || (f32 && (Mz == 768 || Mz == 1024 || Mz == 1152 || Mz == 1536 || Mz == 2048));
+}
+
 // The doubled length of n cells on an axis (-1 beyond the longest).  `blocked`:
 // only the lengths whose y passes also run on a z-blocked workspace.
 inline int mesh_length(int64_t n, int dtype, int axis, bool blocked = false)
@@ -59,15 +65,14 @@ void count_launch();
 // are interleaved (re, im) of the arithmetic type T; source and potential
 // arrays hold IoReal<T>::type (double for df64).
 // `zsh`: the workspace's z planes are grouped in blocks of 2^zsh (w_row in
-// passes.cuh; 0 = plain [Nz][My][Kx]).  Every launch must cover whole blocks
-// (cudaErrorInvalidValue otherwise); plans block the workspace only where the
-// z lines have 2304 points (the paired z pass).
-// Planes per z block of a blocked workspace, as a shift: 16.  The z pass
-// then reads each line group in runs of 16 rows one Kx row (9 KB at 1152^3)
-// apart instead of rows a whole plane (21 MB) apart: 32-byte strided reads
-// measured 3.5 TB/s against 1.5 TB/s, while the y passes' rows move from Kx
-// to 16 Kx apart (4.7 -> 3.2 TB/s on the same read test, on passes that are
-// bound elsewhere).
+// passes.cuh; 0 = plain [Nz][My][Kx]).  A launch on a part of the planes
+// starts at a block.
+// Planes per z block of a blocked workspace, as a shift: 16 (plan_zsh in
+// api.cu says which meshes take it).  The z pass then reads each line group
+// in runs of 16 rows one Kx row (9 KB at 1152^3) apart instead of rows a whole
+// plane (21 MB) apart: 32-byte strided reads measured 3.5 TB/s against 1.5
+// TB/s.  Blocks of 4 and 8 planes measured the same within 1 % (36.2 ms
+// against 37.1 and 37.2 for K3 at 1152^3).
 constexpr int kZBlockShift = 4;
 template <typename T>
 cudaError_t launch_x_forward(int L, const typename IoReal<T>::type *src, void *W, const void *tw, const void *rtw,

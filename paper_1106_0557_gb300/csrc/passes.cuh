@@ -54,9 +54,9 @@ __host__ __device__ __forceinline__ size_t w_row(int64_t z, int64_t y, int64_t M
     if (zsh == 0) return (size_t)(z * My + y);  // (a uniform branch: the plain layout's arithmetic)
     return (size_t)((((z >> zsh) * My + y) << zsh) + (z & ((int64_t(1) << zsh) - 1)));
 }
-// A launch on nz planes of a z-blocked workspace covers whole blocks only
-// (the map above leaves the allocation otherwise).
-inline bool w_blocks_ok(int64_t nz, int zsh) { return zsh >= 0 && zsh <= 6 && (nz & ((int64_t(1) << zsh) - 1)) == 0; }
+// (A z-blocked workspace is allocated in whole blocks; its last block may hold
+// planes past the mesh, which no pass writes and the z pass masks.)
+inline int64_t w_blocks(int64_t nz, int zsh) { return (nz + (int64_t(1) << zsh) - 1) >> zsh; }
 
 // Asynchronous global -> shared copies (cp.async): BYTES = 4, 8 or 16;
 // when `valid` is false nothing is read and the slot is zero-filled.
@@ -789,8 +789,9 @@ struct ZXch {
     Cx<T> *a;  // DB: the second buffer follows at a + L COLS
     int c;
     Hook &hook;
-    int k = 0;  // exchanges done in this tile
-    __device__ __forceinline__ Cx<T> *buf(int i) const { return DB && (i & 1) ? a + (size_t)L * COLS : a; }
+    int flip = 0;  // DB: the buffer of the tile's first exchange
+    int k = 0;     // exchanges done in this tile
+    __device__ __forceinline__ Cx<T> *buf(int i) const { return DB && ((i + flip) & 1) ? a + (size_t)L * COLS : a; }
     __device__ __forceinline__ Cx<T> *free_buf() const { return buf(k); }
     template <int NS, int R>
     __device__ __forceinline__ void exchange(Cx<T> (&v)[E], int t)
@@ -854,13 +855,11 @@ struct ZXch {
 // Nz}) into the other of two staging sets while the CTA transforms the
 // current tile; completion and bounded waits as in the z pass.  Twiddles
 // stay in registers across tiles (lines up to 1024 points), and the
-// exchanges alternate between two buffers where both fit (ZXch).  K2 on the
-// plain workspace with one exchange per transform stages its output tile in
-// the second exchange buffer, which that exchange leaves unused, and thread
-// 0 writes it by tensor stores (tmO: dims {Kx EPC, My, Nz}) after the next
-// tile's first barrier, when every thread has staged its points: the
-// threads issue shared-memory stores instead of global ones (K2 writes
-// twice what it reads).
+// exchanges alternate between two buffers where both fit (ZXch).  K2 stages
+// its output tile in shared memory (YCfg::TSTORE) and thread 0 writes it by
+// tensor stores (tmO: every row y < My) after the next tile's first barrier,
+// when every thread has staged its points: the threads issue shared-memory
+// stores instead of global ones (K2 writes twice what it reads).
 // ---------------------------------------------------------------------
 template <typename T, int L>
 struct YCfg {
@@ -895,7 +894,15 @@ struct YCfg {
     // where it still fits the resident CTAs
     static constexpr bool fits(size_t bytes) { return bytes <= 227 * 1024 && MIN_BLOCKS * (bytes + 1024) <= 228 * 1024; }
     static constexpr bool DBX_F = fits(2 * XCH + 2 * IN_F + 16), DBX_I = fits(2 * XCH + 2 * IN_I + 16);
-    static constexpr size_t SMEM_F = (DBX_F ? 2 : 1) * XCH + 2 * IN_F + 16,
+    // K2's output tile is staged for tensor stores (k_y_pass) in the second
+    // exchange buffer where a transform has one exchange, else (FP32) in a
+    // buffer of its own where that fits
+    static constexpr size_t SMEM_F0 = (DBX_F ? 2 : 1) * XCH + 2 * IN_F + 16;
+    static constexpr bool STAGE_2ND = DBX_F && RadixCount<typename YShape<T, L>::Rad>::value == 2;
+    static constexpr bool STAGE_OWN = !STAGE_2ND && sizeof(T) == 4 && fits(SMEM_F0 + XCH);
+    static constexpr bool TSTORE = STAGE_2ND || STAGE_OWN;
+    static constexpr size_t OFF_STAGE = STAGE_2ND ? XCH : (DBX_F ? 2 : 1) * XCH;
+    static constexpr size_t SMEM_F = SMEM_F0 + (STAGE_OWN ? XCH : 0),
                             SMEM_I = (DBX_I ? 2 : 1) * XCH + 2 * IN_I + 16;
     // twiddles in registers across tiles, except for the long lines, whose
     // per-thread share (29 points for 2304) would spill
@@ -919,10 +926,10 @@ k_y_pass(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtens
     constexpr int NB = FWD ? C::NB_F : C::NB_I, BOX = FWD ? C::BOX_F : C::BOX_I;
     constexpr size_t IN = FWD ? C::IN_F : C::IN_I;
     constexpr bool DBX = FWD ? C::DBX_F : C::DBX_I;
-    constexpr bool TSTORE = FWD && !BLK && DBX && RadixCount<Rad>::value == 2;
+    constexpr bool TSTORE = FWD && C::TSTORE;
     extern __shared__ __align__(128) unsigned char ysmem[];
     Cx<T> *xs = reinterpret_cast<Cx<T> *>(ysmem);            // exchange buffer(s)
-    unsigned char *s_in = ysmem + (DBX ? 2 : 1) * C::XCH;  // [set][row][TX]
+    unsigned char *s_in = ysmem + ((DBX ? 2 : 1) + (FWD && C::STAGE_OWN ? 1 : 0)) * C::XCH;  // [set][row][TX]
     uint64_t *bar = reinterpret_cast<uint64_t *>(s_in + 2 * IN);
     const int tid = threadIdx.x;
     const int c = tid % TX, t = tid / TX;
@@ -953,13 +960,18 @@ k_y_pass(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtens
     auto no_hook = [](int) {};
     typename ZTwiddles<C::TW_REGS, T, L, E, Rad>::type twr;
     twr.load(tw, t);
-    Cx<T> *so = xs + (size_t)L * TX;  // TSTORE: output staging [row][TX], 128-byte aligned
+    Cx<T> *so = reinterpret_cast<Cx<T> *>(ysmem + C::OFF_STAGE);  // TSTORE: output staging [row][TX]
     int prev = -1;                     // TSTORE: the tile whose staged output awaits its stores
     auto store_prev = [&]() {          // thread 0
         const int z = prev / ntx, xt = prev - z * ntx;
 #pragma unroll
-        for (int b = 0; b < C::NB_I; ++b)
-            tma_store_3d(&tmO, so + (size_t)b * C::BOX_I * TX, xt * TX * C::EPC, b * C::BOX_I, z);
+        for (int b = 0; b < C::NB_I; ++b) {
+            const Cx<T> *src = so + (size_t)b * C::BOX_I * TX;
+            if constexpr (!BLK)
+                tma_store_3d(&tmO, src, xt * TX * C::EPC, b * C::BOX_I, z);
+            else  // tmO dims {Kx EPC, 2^zsh, My, blocks}
+                tma_store_4d(&tmO, src, xt * TX * C::EPC, z & ((1 << zsh) - 1), b * C::BOX_I, z >> zsh);
+        }
         bulk_commit();
     };
     int tile = blockIdx.x, it = 0;
@@ -1035,12 +1047,15 @@ k_y_pass(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtens
 // staged, [z < L/2][IS] (IS = TX, or 2 TX where a box holds two tiles),
 // offset to the tile's first column; `sg`: the spectrum block of the
 // thread's line, [kz'][TX].  `before_g` runs before the spectrum is read and
-// returns false (the same on every thread) to abandon the tile.
-template <typename T, int L, int IS, bool SYNC_ALL = false, typename SH = ZShape<T, L>, typename TWR, typename Xch,
-          typename BeforeG>
+// returns false (the same on every thread) to abandon the tile.  `staged`:
+// where the result goes for the caller's tensor stores, [g][z < L/2][TX]
+// (null: the threads store it themselves).
+template <typename T, int L, int IS, bool SYNC_ALL = false, typename SH = ZShape<T, L>, int ZSH = 0, typename TWR,
+          typename Xch, typename BeforeG>
 __device__ __forceinline__ bool z_tile(const Cx<T> *sin, const T *sg, int pr, int xt, Cx<T> *__restrict__ W,
-                                       const T *__restrict__ Gs, T gscale, int Nz, int My, int Kx, int zsh, int c,
-                                       int g, int t, const TWR &twr, const Cx<T> *twz, Xch &xch, BeforeG before_g)
+                                       const T *__restrict__ Gs, T gscale, int Nz, int My, int Kx, int c, int g,
+                                       int t, const TWR &twr, const Cx<T> *twz, Xch &xch, BeforeG before_g,
+                                       Cx<T> *staged = nullptr)
 {
     using C = ZCfg<T, L, SH>;
     using Rad = typename SH::Rad;
@@ -1056,6 +1071,12 @@ __device__ __forceinline__ bool z_tile(const Cx<T> *sin, const T *sg, int pr, in
     Cx<T> v[E];
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = m < E / 2 ? sin[m * NT * IS] : Cx<T>{(T)0, (T)0};
+    if (ZSH > 0 && (Nz & ((1 << ZSH) - 1))) {
+        // planes of the last block past the mesh hold nothing
+#pragma unroll
+        for (int m = 0; m < E / 2; ++m)
+            if (t + m * NT >= Nz) v[m] = {(T)0, (T)0};
+    }
 
     z_fft<C::TWR, true, T, L, E>(v, t, twr, twz, xch, Rad{});
     if (!before_g()) return false;
@@ -1098,23 +1119,21 @@ __device__ __forceinline__ bool z_tile(const Cx<T> *sin, const T *sg, int pr, in
 #pragma unroll
     for (int m = 0; m < E; ++m) v[m] = cswap(v[m]);
     z_fft<C::TWR, false, T, L, E>(v, t, twr, twz, xch, Rad{});
-    if (active && zsh == 0) {
-        Cx<T> *base = W + (size_t)ky * Kx + kx;
-        const size_t zstride = (size_t)My * Kx;
+    if (staged) {
+        // [g][z < Lh][TX] for the tile's tensor stores
+        Cx<T> *so = staged + (size_t)(g * Lh + t) * TX + c;
 #pragma unroll
-        for (int m = 0; m < E / 2; ++m) {
-            const int z = t + m * NT;
-            if (z < Nz) base[(size_t)z * zstride] = cswap(v[m]);
-        }
+        for (int m = 0; m < E / 2; ++m) so[m * NT * TX] = cswap(v[m]);
+        fence_async_smem();
     } else if (active) {
-        Cx<T> *base = W + ((size_t)ky << zsh) * Kx + kx;
+        // z = t + m NT: NT is a multiple of the block, so the rows of a thread
+        // lie NT My apart in either layout
+        static_assert(NT % (1 << ZSH) == 0, "a thread's planes step by whole blocks");
+        Cx<T> *base = W + (ZSH ? w_row(t, ky, My, ZSH) : (size_t)t * My + ky) * Kx + kx;
+        const size_t step = (size_t)NT * My * Kx;
 #pragma unroll
-        for (int m = 0; m < E / 2; ++m) {
-            const int z = t + m * NT;
-            // w_row(z, ky) - w_row(0, ky): (z >> zsh) blocks, row z & (2^zsh - 1)
-            const size_t zr = (((size_t)(z >> zsh) * My) << zsh) + (z & ((1 << zsh) - 1));
-            if (z < Nz) base[zr * Kx] = cswap(v[m]);
-        }
+        for (int m = 0; m < E / 2; ++m)
+            if (t + m * NT < Nz) base[m * step] = cswap(v[m]);
     }
     return true;
 }
@@ -1137,8 +1156,16 @@ __device__ __forceinline__ bool z_tile(const Cx<T> *sin, const T *sg, int pr, in
 // copies are issued after the barrier of the tile's first exchange, which
 // every thread reaches after reading its input; the other spectrum set was
 // last read by the previous tile, before the barriers of its transforms.
+//
+// On a z-blocked workspace (ZSH) the result leaves by tensor stores too: the
+// threads stage it in the exchange buffer that the tile's last exchange leaves
+// free, and thread 0 writes it out after the next tile's first barrier, with
+// the map of the loads (planes of the last block past the mesh are written and
+// never used).  K3 at 512^3 1774 -> 1572 us, at 576^3 2799 -> 2566; on plain
+// planes per-thread stores are faster (187 against 189 us at 256^3, 2372
+// against 2904 at 768 x 384 x 384), so those keep them.
 // ---------------------------------------------------------------------
-template <typename T, int L>
+template <typename T, int L, int ZSH = 0>
 __global__ void __launch_bounds__(ZCfg<T, L>::THREADS, ZCfg<T, L>::MIN_BLOCKS)
 k_z_convolve(const __grid_constant__ CUtensorMap tmW, Cx<T> *__restrict__ W, const Cx<T> *__restrict__ tw,
              const T *__restrict__ G, const T *__restrict__ Gs, T gscale, int Nz, int My, int Kx, int ntiles,
@@ -1148,6 +1175,7 @@ k_z_convolve(const __grid_constant__ CUtensorMap tmW, Cx<T> *__restrict__ W, con
     static_assert(C::DBX, "the paired lines take k_z_convolve_pairs");
     constexpr int E = C::E, TX = C::TX, COLS = C::COLS;
     constexpr int Lh = L / 2;
+    constexpr bool TST = ZSH > 0;  // the result leaves by tensor stores
     extern __shared__ __align__(128) unsigned char zsmem[];
     Cx<T> *sm = reinterpret_cast<Cx<T> *>(zsmem);             // two exchange buffers
     unsigned char *s_in = zsmem + C::OFF_IN;                   // [g][z < Lh][TX]
@@ -1191,9 +1219,16 @@ k_z_convolve(const __grid_constant__ CUtensorMap tmW, Cx<T> *__restrict__ W, con
 #pragma unroll
         for (int zb = 0; zb < C::NZB; ++zb) {
             const size_t off = (size_t)zb * C::BOXZ * TX * sizeof(Cx<T>);
-            tma_load_3d(s_in + off, &tmW, xt * TX * C::EPC, pr, zb * C::BOXZ, &bar[0]);
-            tma_load_3d(s_in + C::IN_GROUP + off, &tmW, xt * TX * C::EPC, ky1, zb * C::BOXZ - (C::SHIFT ? 1 : 0),
-                        &bar[0]);
+            if constexpr (ZSH == 0) {
+                tma_load_3d(s_in + off, &tmW, xt * TX * C::EPC, pr, zb * C::BOXZ, &bar[0]);
+                tma_load_3d(s_in + C::IN_GROUP + off, &tmW, xt * TX * C::EPC, ky1, zb * C::BOXZ - (C::SHIFT ? 1 : 0),
+                            &bar[0]);
+            } else {  // tmW dims {Kx EPC, 2^ZSH, My, blocks}, box {TX EPC, 2^ZSH, 1, BOXZ >> ZSH}
+                static_assert(ZSH == 0 || (!C::SHIFT && C::BOXZ % (1 << ZSH) == 0), "boxes of whole blocks");
+                tma_load_4d(s_in + off, &tmW, xt * TX * C::EPC, 0, pr, (zb * C::BOXZ) >> ZSH, &bar[0]);
+                tma_load_4d(s_in + C::IN_GROUP + off, &tmW, xt * TX * C::EPC, 0, ky1, (zb * C::BOXZ) >> ZSH,
+                            &bar[0]);
+            }
         }
         T *gdst = s_g + (size_t)set * 2 * C::GBLK;
         bulk_load(gdst, G + lay.block(pr, xt), (uint32_t)C::G_BLK, &bar[0]);
@@ -1203,6 +1238,21 @@ k_z_convolve(const __grid_constant__ CUtensorMap tmW, Cx<T> *__restrict__ W, con
     using Rad = typename ZShape<T, L>::Rad;
     typename ZTwiddles<C::TWR, T, L, E, Rad>::type twr;  // this thread's twiddles, for every tile (when TW_REGS)
     twr.load(tw, t);
+    // TST: the tile whose staged output awaits its stores (thread 0)
+    int prev = -1;
+    auto staging = [&](int flip) { return sm + (flip ? (size_t)L * COLS : 0); };
+    auto store_prev = [&](int flip) {
+        const int pr = prev / ntx, xt = z_rotate<T>(prev - pr * ntx, pr, ntx);
+#pragma unroll
+        for (int gi = 0; gi < 2; ++gi) {
+            const int ky = gi == 0 ? pr : (pr == 0 ? My / 2 : My - pr);
+#pragma unroll
+            for (int zb = 0; zb < C::NZB; ++zb)
+                tma_store_4d(&tmW, staging(flip) + (size_t)(gi * Lh + zb * C::BOXZ) * TX, xt * TX * C::EPC, 0, ky,
+                             (zb * C::BOXZ) >> ZSH);
+        }
+        bulk_commit();
+    };
     int tile = blockIdx.x, it = 0;
     bool ok = true;
     // test_extra_tx is a test hook: bytes the first tile's barrier expects
@@ -1215,16 +1265,32 @@ k_z_convolve(const __grid_constant__ CUtensorMap tmW, Cx<T> *__restrict__ W, con
         auto hook = [&](int k) {
             if (k == 0 && tid == 0 && next < ntiles) issue(next, set ^ 1, 0u);
         };
-        ZXch<T, L, E, COLS, C::SWZ, true, decltype(hook)> xch{sm, col, hook};
+        // TST: the tile's first exchange takes the buffer that does not hold the
+        // previous tile's staged output; its barrier follows thread 0's wait
+        // until the stores have read that, so the later exchanges may use it
+        const int flip = TST ? it & 1 : 0;
+        ZXch<T, L, E, COLS, C::SWZ, true, decltype(hook), TST> xch{sm, col, hook, flip};
         if (!__syncthreads_and(mbar_wait_bounded(&bar[0], (uint32_t)it & 1u, kCopyWaitNs))) {
             ok = false;
             break;
+        }
+        if constexpr (TST) {
+            if (tid == 0 && prev >= 0) store_prev(flip ^ 1);
         }
         const int pr = tile / ntx, xt = z_rotate<T>(tile - pr * ntx, pr, ntx);
         // line group 1 staged one row later with SHIFT (its row 0 is plane -1)
         const Cx<T> *sin = reinterpret_cast<const Cx<T> *>(s_in + g * C::IN_GROUP) + (C::SHIFT && g ? TX : 0);
         const T *sg = s_g + ((size_t)set * 2 + (pr == 0 ? g : 0)) * C::GBLK;
-        z_tile<T, L, TX>(sin, sg, pr, xt, W, Gs, gscale, Nz, My, Kx, 0, c, g, t, twr, twz, xch, [] { return true; });
+        z_tile<T, L, TX, false, ZShape<T, L>, ZSH>(sin, sg, pr, xt, W, Gs, gscale, Nz, My, Kx, c, g, t, twr, twz, xch,
+                                                   [] { return true; }, TST ? staging(flip) : nullptr);
+        prev = tile;
+    }
+    if constexpr (TST) {
+        __syncthreads();  // every thread has staged the last tile (the exit is uniform)
+        if (tid == 0) {
+            if (prev >= 0) store_prev((it - 1) & 1);
+            bulk_wait_all();
+        }
     }
     if (!ok && tid == 0) {
         // a wait gave up: flag it, then let this tile's copies land (bounded
@@ -1351,8 +1417,8 @@ k_z_convolve_pairs(const __grid_constant__ CUtensorMap tmW, Cx<T> *__restrict__ 
             };
             const Cx<T> *sin = reinterpret_cast<const Cx<T> *>(s_in + g * C::PIN_GROUP) + s * TX;
             const T *sg = s_g + ((size_t)(pr == 0 ? g : 0) * 2 + s) * C::GBLK;
-            if (!z_tile<T, L, PTX>(sin, sg, pr, xt0 + s, W, Gs, gscale, Nz, My, Kx, zsh, c, g, t, twr, twz, xch,
-                                   spectrum_landed)) {
+            if (!z_tile<T, L, PTX, false, ZShape<T, L>, ZSH>(sin, sg, pr, xt0 + s, W, Gs, gscale, Nz, My, Kx, c, g, t,
+                                                             twr, twz, xch, spectrum_landed)) {
                 ok = false;
                 break;
             }

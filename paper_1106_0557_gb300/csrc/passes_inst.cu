@@ -161,7 +161,7 @@ static cudaError_t run_x_forward(const In<T> *src, void *W, const void *tw, cons
     using C = RowCfg<T, L, XShapeF<T, L>>;
     static std::atomic<uint64_t> done{0};
     static std::atomic<int> resident{0};
-    if (Ny <= 0 || nrows % Ny || !w_blocks_ok(nrows / Ny, zsh)) return cudaErrorInvalidValue;
+    if (Ny <= 0 || nrows % Ny) return cudaErrorInvalidValue;
     cudaError_t e = ensure_smem(k_x_forward<T, L>, C::SMEM, done);
     if (e != cudaSuccess) return e;
     const unsigned grid =
@@ -176,7 +176,7 @@ static cudaError_t run_x_inverse(const void *W, In<T> *phi, const void *tw, cons
     using C = RowCfg<T, L>;
     static std::atomic<uint64_t> done{0};
     static std::atomic<int> resident{0};
-    if (Ny <= 0 || nrows % Ny || !w_blocks_ok(nrows / Ny, zsh)) return cudaErrorInvalidValue;
+    if (Ny <= 0 || nrows % Ny) return cudaErrorInvalidValue;
     cudaError_t e = ensure_smem(k_x_inverse<T, L>, C::SMEM, done);
     if (e != cudaSuccess) return e;
     const unsigned grid =
@@ -220,7 +220,7 @@ template cudaError_t ISOFFT_LAUNCHER(launch_x_inverse)<Real>(int, const void *, 
 #endif
 
 #if ISOFFT_GROUP == 2
-constexpr bool kBlocked = ISOFFT_PART == 1;  // mesh_length's `blocked` lengths
+constexpr bool kBlocked = ISOFFT_PART == 1 || ISOFFT_TYPE == 1;  // the lengths z-blocked meshes take
 template <typename T, int L, bool FWD, bool NARROW>
 static cudaError_t run_y_tile(void *W, const void *tw, int Ny, int Kx, int Nz, int zsh, cudaStream_t st)
 {
@@ -230,7 +230,6 @@ static cudaError_t run_y_tile(void *W, const void *tw, int Ny, int Kx, int Nz, i
     if (zsh && !kBlocked) return cudaErrorInvalidValue;
     auto *k = zsh ? (FWD ? k_y_forward<T, L, NARROW, kBlocked> : k_y_inverse<T, L, NARROW, kBlocked>)
                   : (FWD ? k_y_forward<T, L, NARROW, false> : k_y_inverse<T, L, NARROW, false>);
-    if (!w_blocks_ok(Nz, zsh)) return cudaErrorInvalidValue;
     cudaError_t e = ensure_smem(k, C::SMEM, zsh ? doneb : done0);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)((Kx + C::TX - 1) / C::TX), (unsigned)Nz);
@@ -259,13 +258,12 @@ static cudaError_t run_y_stream(void *W, const void *tw, int Ny, int Kx, int Nz,
     // {Kx EPC, 2^zsh, rows, Nz >> zsh}); K2 sees only rows y < Ny
     EncodeTiledFn encode = encode_tiled();
     if (!encode) return cudaErrorNotSupported;
-    if (!w_blocks_ok(Nz, zsh)) return cudaErrorInvalidValue;
     CUtensorMap map;
     const cuuint64_t rows = (cuuint64_t)(FWD ? Ny : L), cb = sizeof(Cx<T>);
     const cuuint64_t dims3[3] = {(cuuint64_t)Kx * C::EPC, rows, (cuuint64_t)Nz};
     const cuuint64_t strides3[2] = {(cuuint64_t)Kx * cb, (cuuint64_t)L * Kx * cb};
     const cuuint32_t box3[3] = {(cuuint32_t)(C::TX * C::EPC), (cuuint32_t)(FWD ? C::BOX_F : C::BOX_I), 1u};
-    const cuuint64_t dims4[4] = {(cuuint64_t)Kx * C::EPC, (cuuint64_t)1 << zsh, rows, (cuuint64_t)(Nz >> zsh)};
+    const cuuint64_t dims4[4] = {(cuuint64_t)Kx * C::EPC, (cuuint64_t)1 << zsh, rows, (cuuint64_t)w_blocks(Nz, zsh)};
     const cuuint64_t strides4[3] = {(cuuint64_t)Kx * cb, ((cuuint64_t)Kx * cb) << zsh,
                                     ((cuuint64_t)L * Kx * cb) << zsh};
     const cuuint32_t box4[4] = {(cuuint32_t)(C::TX * C::EPC), 1u, (cuuint32_t)(FWD ? C::BOX_F : C::BOX_I), 1u};
@@ -274,14 +272,17 @@ static cudaError_t run_y_stream(void *W, const void *tw, int Ny, int Kx, int Nz,
                zsh ? box4 : box3, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
-    // K2's output map on the plain workspace (every row y < My), for the
-    // kernels that write their tiles by tensor stores; elsewhere unused
+    // K2's output map (every row y < My), for the kernels that write their
+    // tiles by tensor stores; elsewhere unused
     CUtensorMap omap = map;
-    if (FWD && !zsh) {
-        const cuuint64_t odims[3] = {(cuuint64_t)Kx * C::EPC, (cuuint64_t)L, (cuuint64_t)Nz};
-        const cuuint32_t obox[3] = {(cuuint32_t)(C::TX * C::EPC), (cuuint32_t)C::BOX_I, 1u};
-        if (encode(&omap, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, W, odims, strides3, obox, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+    if (FWD && C::TSTORE) {
+        const cuuint64_t odims3[3] = {(cuuint64_t)Kx * C::EPC, (cuuint64_t)L, (cuuint64_t)Nz};
+        const cuuint32_t obox3[3] = {(cuuint32_t)(C::TX * C::EPC), (cuuint32_t)C::BOX_I, 1u};
+        const cuuint64_t odims4[4] = {dims4[0], dims4[1], (cuuint64_t)L, dims4[3]};
+        const cuuint32_t obox4[4] = {(cuuint32_t)(C::TX * C::EPC), 1u, (cuuint32_t)C::BOX_I, 1u};
+        if (encode(&omap, CU_TENSOR_MAP_DATA_TYPE_UINT64, zsh ? 4 : 3, W, zsh ? odims4 : odims3,
+                   zsh ? strides4 : strides3, zsh ? obox4 : obox3, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                   CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
     }
@@ -339,26 +340,24 @@ static cudaError_t run_z(void *W, const void *tw, const T *G, const T *Gs, T gsc
                          int zsh, unsigned *status, unsigned test_extra_tx, cudaStream_t st)
 {
     using C = ZCfg<T, L>;
-    // the paired form comes in a plain and a z-blocked instance
+    // a plain and, on the lengths that meshes block, a z-blocked instance
+    constexpr int ZB = z_blocks(L, sizeof(T) == 4) ? kZBlockShift : 0;
     constexpr auto kernel0 = []() {
         if constexpr (C::DBX)
-            return k_z_convolve<T, L>;
+            return k_z_convolve<T, L, 0>;
         else
             return k_z_convolve_pairs<T, L, 0>;
     }();
     constexpr auto kernelb = []() {
         if constexpr (C::DBX)
-            return k_z_convolve<T, L>;
+            return k_z_convolve<T, L, ZB>;
         else
-            return k_z_convolve_pairs<T, L, L == 2304 ? kZBlockShift : 0>;
+            return k_z_convolve_pairs<T, L, ZB>;
     }();
     static std::atomic<uint64_t> done0{0}, doneb{0};
     static std::atomic<int> slots0{0}, slotsb{0};
     if (((uintptr_t)W & 15) || ((uintptr_t)G & 15)) return cudaErrorMisalignedAddress;
-    // the z-blocked workspace is read by the paired form only, in boxes of
-    // whole blocks
-    if (!w_blocks_ok(Nz, zsh) || (zsh && (L != 2304 || C::DBX || zsh != kZBlockShift || C::BOXZ % (1 << zsh))))
-        return cudaErrorInvalidValue;
+    if (zsh && zsh != ZB) return cudaErrorInvalidValue;
     const auto kernel = zsh ? kernelb : kernel0;
     cudaError_t e = ensure_smem(kernel, C::SMEM, zsh ? doneb : done0);
     if (e != cudaSuccess) return e;
@@ -380,7 +379,7 @@ static cudaError_t run_z(void *W, const void *tw, const T *G, const T *Gs, T gsc
     const cuuint64_t strides3[2] = {(cuuint64_t)Kx * cb, (cuuint64_t)My * Kx * cb};
     const cuuint32_t box3[3] = {bx, 1u, (cuuint32_t)C::BOXZ};
     const cuuint64_t dims4[4] = {(cuuint64_t)Kx * C::EPC, (cuuint64_t)1 << zsh, (cuuint64_t)My,
-                                 (cuuint64_t)(Nz >> zsh)};
+                                 (cuuint64_t)w_blocks(Nz, zsh)};
     const cuuint64_t strides4[3] = {(cuuint64_t)Kx * cb, ((cuuint64_t)Kx * cb) << zsh,
                                     ((cuuint64_t)My * Kx * cb) << zsh};
     const cuuint32_t box4[4] = {bx, 1u << zsh, 1u, (cuuint32_t)(C::BOXZ >> zsh)};
