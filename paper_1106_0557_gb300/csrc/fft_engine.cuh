@@ -843,14 +843,17 @@ template <>
 struct ZShape<double, 768> : ZShape16B768 {};
 template <>
 struct ZShape<df64, 768> : ZShape16B768 {};
-// 2304-point lines (and FP32 lines of 1296 points, at 36 points a thread: 469
-// us against 577 at 1536) read their twiddles from the table (a thread's share
-// would not fit in registers next to its points).  FP32 takes 24 points per
-// thread and three stages, so that a tile of two columns (16 bytes, the
-// narrowest tensor-copy row) fits 384 threads; 16-byte FP64-class points
-// keep 12 per thread on one-column tiles.  (48 points a thread in two
-// stages, as the y passes take, measured 11 % slower here: 192 threads, 6
-// warps per SM.)
+// FP64-class 2304-point lines (and FP32 lines of 1296 points, at 36 points a
+// thread: 469 us against 577 at 1536) read their twiddles from the table (a
+// thread's share would not fit in registers next to its points).  FP32 takes
+// 24 points per thread and three stages, so that a tile of two columns (16
+// bytes, the narrowest tensor-copy row) fits 384 threads; in the order
+// 24 4 24 the thread count is a multiple of every stage's stride and 26
+// twiddles serve all its butterflies from registers (24 24 4 read 41 a
+// transform from shared memory: K3 at 1152^3 36.2 -> 34.2 ms).  16-byte
+// FP64-class points keep 12 per thread on one-column tiles.  (48 points a
+// thread in two stages, as the y passes take, measured 11 % slower here: 192
+// threads, 6 warps per SM.)
 template <typename T>
 struct ZShape<T, 2304> : Shape<T, 2304> {
     static constexpr bool TW_REGS = false;
@@ -864,8 +867,8 @@ struct ZShape<float, 1296> {
 template <>
 struct ZShape<float, 2304> {
     static constexpr int E = 24;
-    using Rad = Radices<24, 24, 4>;
-    static constexpr bool TW_REGS = false;
+    using Rad = Radices<24, 4, 24>;
+    static constexpr bool TW_REGS = true;
 };
 
 // The x passes hold one row per (half) warp; a 256-point FP32 row runs 16
