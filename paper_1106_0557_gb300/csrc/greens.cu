@@ -21,30 +21,47 @@
 
 namespace isofft {
 
-static __global__ void k_green_octant(double *__restrict__ g, int X, int Y, int Z, double hx, double hy,
-                                      double hz)
+// 1 / sqrt(x): the float unit's estimate (about 2^-22) and one step of
+// Householder's third-order iteration, w (1 + e/2 + 3 e^2/8) with e = 1 - x w^2
+// (error e^3), in eight FP64 operations; the library call outside float range.
+static __device__ __forceinline__ double inv_sqrt(double x)
 {
-    const int64_t n = (int64_t)X * Y * Z;
+    if (!(x < 1e37 && x > 1e-37)) return rsqrt(x);
+    const double w = (double)rsqrtf((float)x);
+    const double e = fma(-x * w, w, 1.0);
+    return fma(w * e, fma(0.375, e, 0.5), w);
+}
+
+// A thread takes one (x, y) and `zc` planes; block row blockIdx.y.  Bound by
+// FP64 arithmetic: the quotient by the square root with 64-bit indices took
+// 22.9 us on a 65^3 octant, this 16.8 us (0.82 -> 0.52 ms at 257^3).
+static __global__ void k_green_octant(double *__restrict__ g, int X, int Y, int Z, double hx, double hy,
+                                      double hz, int zc)
+{
+    grid_wait();
+    const int xy = blockIdx.x * blockDim.x + threadIdx.x;
+    if (xy >= X * Y) return;
+    const int y = xy / X, x = xy - y * X;
     const double num = -hx * hy * hz / (4.0 * 3.14159265358979323846);
     const double hmin = fmin(hx, fmin(hy, hz));
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t x = i % X, y = (i / X) % Y, z = i / ((int64_t)X * Y);
-        double v;
-        if (x == 0 && y == 0 && z == 0) {
-            v = num / hmin;  // Eq. 9: the largest off-origin magnitude
-        } else {
-            const double dx = hx * (double)x, dy = hy * (double)y, dz = hz * (double)z;
-            v = num / sqrt(dx * dx + dy * dy + dz * dz);  // Eq. 6
-        }
-        g[i] = v;
+    const double dx = hx * (double)x, dy = hy * (double)y;
+    const int z1 = min((int)(blockIdx.y + 1) * zc, Z);
+    for (int z = blockIdx.y * zc; z < z1; ++z) {
+        const double dz = hz * (double)z;
+        // Eq. 6; at the origin Eq. 9: the largest off-origin magnitude
+        const double v = xy == 0 && z == 0 ? num / hmin : num * inv_sqrt(fma(dz, dz, fma(dx, dx, dy * dy)));
+        g[(int64_t)z * X * Y + xy] = v;
     }
 }
 
 // One axis of the octant transform, in place: line (a, c) of the octant,
 // elements base[q Cc] (q <= L/2, base = oct + a (L/2 + 1) Cc + c), is
 // mirrored to L points, transformed, and bins 0..L/2 (real) are written back.
-// Lines are grouped NL per CTA (one row buffer each, as the x passes use).
+// The transform of a real even line is real, so two neighbouring lines go
+// through one complex transform as its real and imaginary parts: the pass is
+// bound by FP64 arithmetic, and this halves it (22.2 -> 15.2 us an axis at
+// 65^3, 1.40 -> 0.82 ms at 257^3).
+// Line pairs are grouped NL per CTA (one row buffer each, as the x passes use).
 template <int L>
 struct DctCfg {
     using SH = Shape<double, L>;
@@ -63,27 +80,32 @@ k_cos_lines(double *__restrict__ oct, const Cx<double> *__restrict__ tw, int64_t
     extern __shared__ __align__(16) unsigned char dct_smem[];
     Cx<double> *row = reinterpret_cast<Cx<double> *>(dct_smem) + (threadIdx.x / NT) * RowPad<double, L>::LP;
     const int l = threadIdx.x / NT, t = threadIdx.x % NT;
-    const int64_t lines = A * Cc;
-    for (int64_t l0 = (int64_t)blockIdx.x * C::NL; l0 < lines; l0 += (int64_t)gridDim.x * C::NL) {
-        const int64_t line = l0 + l;
-        const bool active = line < lines;
-        const int64_t a = active ? line / Cc : 0, c = active ? line % Cc : 0;
-        double *base = oct + a * n * Cc + c;
+    const int64_t lines = A * Cc, pairs = (lines + 1) / 2;
+    grid_wait();
+    for (int64_t p0 = (int64_t)blockIdx.x * C::NL; p0 < pairs; p0 += (int64_t)gridDim.x * C::NL) {
+        const int64_t line = 2 * (p0 + l);
+        const bool act0 = line < lines, act1 = line + 1 < lines;
+        const int64_t a = act0 ? line / Cc : 0, c = act0 ? line % Cc : 0;
+        double *base0 = oct + a * n * Cc + c;
+        double *base1 = c + 1 < Cc ? base0 + 1 : oct + (a + 1) * n * Cc;  // line + 1
         Cx<double> v[E];
 #pragma unroll
         for (int m = 0; m < E; ++m) {
             const int p = t + m * NT;
-            const int q = p <= L / 2 ? p : L - p;
-            v[m] = {active ? base[(int64_t)q * Cc] : 0.0, 0.0};
+            const int64_t q = (int64_t)(p <= L / 2 ? p : L - p) * Cc;
+            v[m] = {act0 ? base0[q] : 0.0, act1 ? base1[q] : 0.0};
         }
-        // every thread has read its line before the first exchange's barrier,
+        // every thread has read its lines before the first exchange's barrier,
         // and writes after the last one
         RowXch<double, L, E> xch{row};
         run_stages<double, L, E, false>(v, t, tw, xch, typename C::SH::Rad{});
 #pragma unroll
         for (int m = 0; m < E; ++m) {
             const int k = t + m * NT;
-            if (active && k <= L / 2) base[(int64_t)k * Cc] = v[m].x;
+            if (k <= L / 2) {
+                if (act0) base0[(int64_t)k * Cc] = v[m].x;
+                if (act1) base1[(int64_t)k * Cc] = v[m].y;
+            }
         }
     }
 }
@@ -96,15 +118,13 @@ template <int L>
 static cudaError_t run_cos_lines(double *oct, const Cx<double> *tw, int64_t A, int64_t Cc, cudaStream_t st)
 {
     using C = DctCfg<L>;
-    const int64_t groups = (A * Cc + C::NL - 1) / C::NL;
+    const int64_t groups = ((A * Cc + 1) / 2 + C::NL - 1) / C::NL;
     const int grid = (int)(groups < 152 * 8 ? groups : 152 * 8);
     if (C::SMEM > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k_cos_lines<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
         if (e != cudaSuccess) return e;
     }
-    k_cos_lines<L><<<grid, C::THREADS, C::SMEM, st>>>(oct, tw, A, Cc);
-    count_launch();
-    return cudaGetLastError();
+    return launch_pass(k_cos_lines<L>, dim3(grid), C::THREADS, C::SMEM, st, oct, tw, A, Cc);
 }
 
 // Cosine transform of every octant line along one axis of length M (one of
@@ -141,6 +161,7 @@ static __global__ void k_pack(const double *__restrict__ oct, T *__restrict__ G,
 {
     const int Kx = X - 1;
     const int64_t tot = (int64_t)Y * ntx * blk;
+    grid_wait();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < tot;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int j = (int)(i % blk);
@@ -252,9 +273,8 @@ static cudaError_t pack_spectrum(const int64_t M[3], const double *oct, T *G, T 
     const int tx = z_tile_for<T>((int)M[2]);
     const int ntx = (int)((M[0] / 2 + tx - 1) / tx);
     const int blk = z_spec_block(tx, Z, (int)sizeof(T));
-    k_pack<T><<<grid_for((int64_t)Y * ntx * blk), 256, 0, st>>>(oct, G, Gs, X, Y, Z, tx, ntx, blk, scale);
-    count_launch();
-    return cudaGetLastError();
+    return launch_pass(k_pack<T>, dim3(grid_for((int64_t)Y * ntx * blk)), 256, 0, st, oct, G, Gs, X, Y, Z, tx, ntx, blk,
+                       scale);
 }
 
 // The octant of Eq. 9 (FP64), its three axis transforms in place, the pack.
@@ -264,15 +284,15 @@ static cudaError_t spectrum_steps(const int64_t M[3], const double hn[3], T *G, 
                                   const double *tws, cudaStream_t st)
 {
     const int X = (int)(M[0] / 2 + 1), Y = (int)(M[1] / 2 + 1), Z = (int)(M[2] / 2 + 1);
-    const int64_t n = (int64_t)X * Y * Z;
     if ((reinterpret_cast<uintptr_t>(tws) & 15) || (reinterpret_cast<uintptr_t>(oct) & 7))
         return cudaErrorMisalignedAddress;  // complex-double tables need 16-byte alignment
-    k_green_octant<<<grid_for(n), 256, 0, st>>>(oct, X, Y, Z, hn[0], hn[1], hn[2]);
-    count_launch();
+    const int zc = Z > 128 ? 8 : 2;
+    cudaError_t e = launch_pass(k_green_octant, dim3((unsigned)((X * Y + 255) / 256), (unsigned)((Z + zc - 1) / zc)), 256,
+                                0, st, oct, X, Y, Z, hn[0], hn[1], hn[2], zc);
     const Cx<double> *tw[3] = {reinterpret_cast<const Cx<double> *>(tws),
                                reinterpret_cast<const Cx<double> *>(tws) + M[0],
                                reinterpret_cast<const Cx<double> *>(tws) + M[0] + M[1]};
-    cudaError_t e = cos_transform(M, oct, tw, st);
+    if (e == cudaSuccess) e = cos_transform(M, oct, tw, st);
     if (e == cudaSuccess) e = pack_spectrum<T>(M, oct, G, Gs, st);
     return e;
 }
@@ -306,42 +326,47 @@ cudaError_t build_green_spectrum(const int64_t M[3], const double hn[3], T *G, T
 
 // Same spectrum as build_green_spectrum, enqueued on `st` without allocating
 // or synchronising: the FP64 octant lives in the caller's `oct` scratch
-// (green_octant_elems(M) doubles), the root tables in `ct`
-// (green_cos_elems(M) doubles, computed on the device by k_axis_roots).
-static __global__ void k_axis_roots(double *__restrict__ ct, int mx, int my, int mz)
+// (green_octant_elems(M) doubles), the FP64 root tables in `ct`
+// (green_cos_elems(M) doubles).  k_tables computes these and, from the same
+// roots, the solve's own tables: tw_x = W_Lx^k = W_Mx^2k and rtw = W_Mx^k for
+// k < Lx = Mx/2, tw_y = W_My^k, tw_z = W_Mz^k.
+template <typename T>
+static __global__ void k_tables(double *__restrict__ ct, Cx<T> *__restrict__ tw_x, Cx<T> *__restrict__ rtw,
+                                Cx<T> *__restrict__ tw_y, Cx<T> *__restrict__ tw_z, int mx, int my, int mz)
 {
+    grid_wait();
     const int tot = mx + my + mz;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < tot; i += gridDim.x * blockDim.x) {
-        int k = i, m = mx;
-        if (k >= mx) {
-            k -= mx;
-            m = my;
-            if (k >= my) {
-                k -= my;
-                m = mz;
-            }
-        }
+        const int axis = i < mx ? 0 : (i < mx + my ? 1 : 2);
+        const int k = axis == 0 ? i : (axis == 1 ? i - mx : i - mx - my);
+        const int m = axis == 0 ? mx : (axis == 1 ? my : mz);
         double sn, cs;
         sincospi(2.0 * (double)k / (double)m, &sn, &cs);
         ct[2 * i] = cs;
         ct[2 * i + 1] = -sn;
+        const Cx<T> w = {(T)cs, (T)-sn};
+        if (axis == 0) {
+            if (k < mx / 2) rtw[k] = w;
+            if ((k & 1) == 0) tw_x[k / 2] = w;
+        } else {
+            (axis == 1 ? tw_y : tw_z)[k] = w;
+        }
     }
 }
 
 template <typename T>
-cudaError_t enqueue_green_spectrum(const int64_t M[3], const double hn[3], T *G, T *Gs, double *oct,
-                                   double *ct, cudaStream_t st)
+cudaError_t enqueue_green_spectrum(const int64_t M[3], const double hn[3], T *G, T *Gs, double *oct, double *ct,
+                                   void *tw_x, void *rtw, void *tw_y, void *tw_z, cudaStream_t st)
 {
-    k_axis_roots<<<grid_for(M[0] + M[1] + M[2]), 256, 0, st>>>(ct, (int)M[0], (int)M[1], (int)M[2]);
-    count_launch();
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_pass(k_tables<T>, dim3(grid_for(M[0] + M[1] + M[2])), 256, 0, st, ct, (Cx<T> *)tw_x,
+                                (Cx<T> *)rtw, (Cx<T> *)tw_y, (Cx<T> *)tw_z, (int)M[0], (int)M[1], (int)M[2]);
     if (e == cudaSuccess) e = spectrum_steps<T>(M, hn, G, Gs, oct, ct, st);
     return e;
 }
 template cudaError_t enqueue_green_spectrum<float>(const int64_t *, const double *, float *, float *, double *,
-                                                   double *, cudaStream_t);
-template cudaError_t enqueue_green_spectrum<double>(const int64_t *, const double *, double *, double *,
-                                                    double *, double *, cudaStream_t);
+                                                   double *, void *, void *, void *, void *, cudaStream_t);
+template cudaError_t enqueue_green_spectrum<double>(const int64_t *, const double *, double *, double *, double *,
+                                                    double *, void *, void *, void *, void *, cudaStream_t);
 
 template cudaError_t build_green_spectrum<float>(const int64_t *, const double *, float *, float *,
                                                  cudaStream_t);

@@ -155,10 +155,12 @@ cudaError_t build_green_spectrum(const int64_t M[3], const double hn[3], T *G, T
 // The same spectrum enqueued without allocating or synchronising, in caller
 // scratch: `oct` holds green_octant_elems(M) doubles (the FP64 octant,
 // transformed in place), `ct` holds green_cos_elems(M) doubles (the root
-// tables of the three axes, computed on the device).
+// tables of the three axes, computed on the device).  The solve's root tables
+// (complex T: tw_x and rtw of Mx/2 points, tw_y of My, tw_z of Mz) are filled
+// by the same launch.
 template <typename T>
-cudaError_t enqueue_green_spectrum(const int64_t M[3], const double hn[3], T *G, T *Gs, double *oct,
-                                   double *ct, cudaStream_t st);
+cudaError_t enqueue_green_spectrum(const int64_t M[3], const double hn[3], T *G, T *Gs, double *oct, double *ct,
+                                   void *tw_x, void *rtw, void *tw_y, void *tw_z, cudaStream_t st);
 int64_t green_octant_elems(const int64_t M[3]);
 int64_t green_cos_elems(const int64_t M[3]);
 

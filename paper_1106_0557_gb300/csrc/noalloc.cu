@@ -25,16 +25,6 @@ namespace isofft {
 constexpr size_t kNoallocScratchBytes = 64ull << 20;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes];
 
-template <typename T>
-static __global__ void k_roots(Cx<T> *__restrict__ out, int n, int count)
-{
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < count; k += gridDim.x * blockDim.x) {
-        double s, c;
-        sincospi(2.0 * (double)k / (double)n, &s, &c);
-        out[k] = {(T)c, (T)-s};
-    }
-}
-
 namespace {
 
 std::mutex g_noalloc_mu;
@@ -109,19 +99,11 @@ int solve_noalloc(const int64_t N[3], const int64_t M[3], const double hn[3], do
     const int Nx = (int)N[0], Ny = (int)N[1], Nz = (int)N[2];
     const int Lx = (int)(M[0] / 2), My = (int)M[1], Mz = (int)M[2];
 
-    // tables: W_Lx^k, W_Mx^k (k < Lx), W_My^k, W_Mz^k
-    k_roots<T><<<(Lx + 255) / 256, 256, 0, st>>>(tw_x, Lx, Lx);
-    count_launch();
-    k_roots<T><<<(Lx + 255) / 256, 256, 0, st>>>(rtw, 2 * Lx, Lx);
-    count_launch();
-    k_roots<T><<<(My + 255) / 256, 256, 0, st>>>(tw_y, My, My);
-    count_launch();
-    k_roots<T><<<(Mz + 255) / 256, 256, 0, st>>>(tw_z, Mz, Mz);
-    count_launch();
-    // the spectrum, built in the workspace region before the workspace is used
+    // the tables and the spectrum, built in the workspace region before the
+    // workspace is used
     double *oct = (double *)W;
     double *ct = oct + green_octant_elems(M);
-    e = enqueue_green_spectrum<T>(M, hn, G, Gs, oct, ct, st);
+    e = enqueue_green_spectrum<T>(M, hn, G, Gs, oct, ct, tw_x, rtw, tw_y, tw_z, st);
     if (e == cudaSuccess)
         e = launch_x_forward<T>(Lx, (const T *)src, W, tw_x, rtw, Nx, Ny, My, (int64_t)Ny * Nz, 0, st);
     if (e == cudaSuccess) e = launch_y_forward<T>(My, W, tw_y, Ny, Lx, Nz, 0, (unsigned *)b, y_default_variant(My, sizeof(T)), st);

@@ -44,6 +44,35 @@
 
 namespace isofft {
 
+// Launch with the programmatic-serialization attribute: the launch is
+// processed while the stream's previous kernel still runs, its CTAs start as
+// that kernel's last ones leave, and each waits in grid_wait() before it
+// touches the previous results.  Without it every pass of a small solve paid
+// about 2 us between kernels: solves back to back in one stream took 24.9 us
+// at FP32 64^3 (17.2 now), 28.0 at 100 x 70 x 30 (17.7), 70.0 at 128^3 (57.0),
+// 416 at 256^3 (404.5).  The kernels do not trigger their successors early
+// (griddepcontrol.launch_dependents): CTAs that sit waiting hold the SM room
+// that solves on other streams could use (64 grids on eight streams 942-960
+// us with triggers at the start or end of each CTA, 922-930 without, 935
+// before).
+template <typename... K, typename... A>
+inline cudaError_t launch_pass(void (*kernel)(K...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, K(args)...);
+    count_launch();
+    return e;
+}
+
 // Row (z, y) of the workspace W, in complex elements / Kx.  With zsh > 0 the
 // planes are grouped in blocks of 2^zsh: [z >> zsh][My][z & (2^zsh - 1)][Kx],
 // so that the z lines of one (kx, ky) lie 2^zsh rows apart within a block
