@@ -217,6 +217,21 @@ struct RowCfg {
     // table in every stage: FP32 forward rows of 192 and 384 points, inverse
     // rows of 128, 384, 768 and 1152.  Elsewhere the extra registers cost
     // more occupancy than the table reads do.
+    // CTAs per SM that FP32 rows' registers are capped for (K1: MIN_F, K5:
+    // MIN_I; 0: no cap) where the compiler takes a few more than the next step
+    // of the occupancy allows: K1 on 768-point rows 438 us at 84 registers (two
+    // CTAs), 384 at 80 (three) at 768 x 384 x 384.
+    static constexpr int min_f()
+    {
+        if (sizeof(T) != 4) return 0;
+        return L == 48 ? 5 : L == 64 ? 6 : L == 162 ? 4 : (L == 288 || L == 576 || L == 768) ? 3 : L == 648 ? 2 : 0;
+    }
+    static constexpr int min_i()
+    {
+        if (sizeof(T) != 4) return 0;
+        return L == 48 ? 5 : (L == 64 || L == 512) ? 6 : L == 648 ? 2 : 0;
+    }
+    static constexpr int MIN_F = min_f(), MIN_I = min_i();
     static constexpr bool TWR_F = sizeof(T) == 4 && (L == 192 || L == 384);
     static constexpr bool TWR_I = sizeof(T) == 4 && (L == 128 || L == 384 || L == 768 || L == 1152);
 };
@@ -715,7 +730,7 @@ __device__ __forceinline__ void y_inverse_tile(Cx<T> *__restrict__ W, const Cx<T
 // every CTA takes one group.
 // ---------------------------------------------------------------------
 template <typename T, int L>
-__global__ void __launch_bounds__(RowCfg<T, L, XShapeF<T, L>>::THREADS)
+__global__ void __launch_bounds__(RowCfg<T, L, XShapeF<T, L>>::THREADS, RowCfg<T, L, XShapeF<T, L>>::MIN_F)
 k_x_forward(const In<T> *__restrict__ src, Cx<T> *__restrict__ W, const Cx<T> *__restrict__ tw,
             const Cx<T> *__restrict__ rtw, int Nx, int Ny, int My, int64_t nrows, int zsh)
 {
@@ -747,7 +762,7 @@ k_x_forward(const In<T> *__restrict__ src, Cx<T> *__restrict__ W, const Cx<T> *_
 }
 
 template <typename T, int L>
-__global__ void __launch_bounds__(RowCfg<T, L>::THREADS)
+__global__ void __launch_bounds__(RowCfg<T, L>::THREADS, RowCfg<T, L>::MIN_I)
 k_x_inverse(const Cx<T> *__restrict__ W, In<T> *__restrict__ phi, const Cx<T> *__restrict__ tw,
             const Cx<T> *__restrict__ rtw, int Nx, int Ny, int My, int64_t nrows, int zsh)
 {
