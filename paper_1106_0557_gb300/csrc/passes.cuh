@@ -304,7 +304,8 @@ constexpr int z_tile_width(int rb, int nt, int L, int e)
 constexpr int z_min_blocks(int rb, int nt, int L, int e, int tx)
 {
     if (rb == 8 && e == 12 && nt >= 32 && nt <= 64) return 384 / (2 * tx * nt);
-    if (rb == 8) return 2 * tx * nt <= 192 && 2 * (z_smem(tx, L, rb) + 1024) <= 228 * 1024 ? 2 : 1;
+    if (rb == 8)
+        return 2 * tx * nt <= 192 && 2 * (z_smem(tx, L, rb) + 1024) <= 228 * 1024 ? 2 : 1;
     const int threads = 2 * tx * nt, want = (e <= 16 ? 512 : 384) / threads;
     const int fit = (int)((size_t)228 * 1024 / (z_smem_dbx(tx, L, rb) + 1024));
     const int n = want < fit ? want : fit;
@@ -355,7 +356,10 @@ struct ZCfg {
     // shared memory (read by every stage, loaded once per CTA)
     static constexpr bool TWR = SH::TW_REGS;
     static constexpr size_t TWS = TWR ? 0 : (size_t)L * sizeof(Cx<T>);
-    static constexpr int MIN_BLOCKS = z_min_blocks((int)sizeof(T), NT, L, E, TX);
+    // (float pairs at 256 points: two CTAs of 128 registers, 157.6 -> 142.6 us at
+    // 128^3; FP64 there 761 -> 778, and 128 and 64 points no faster)
+    static constexpr int MIN_BLOCKS =
+        std::is_same<T, df64>::value && L == 256 ? 2 : z_min_blocks((int)sizeof(T), NT, L, E, TX);
     // Two exchange buffers used in turn need one CTA barrier per exchange
     // instead of two; the input is then staged once per tile (the next
     // tile's copies start after the first exchange's barrier, when every
