@@ -306,7 +306,7 @@ constexpr int z_min_blocks(int rb, int nt, int L, int e, int tx)
     if (rb == 8 && e == 12 && nt >= 32 && nt <= 64) return 384 / (2 * tx * nt);
     if (rb == 8)
         return 2 * tx * nt <= 192 && 2 * (z_smem(tx, L, rb) + 1024) <= 228 * 1024 ? 2 : 1;
-    const int threads = 2 * tx * nt, want = (e <= 16 ? 512 : 384) / threads;
+    const int threads = 2 * tx * nt, want = (e <= 8 ? 768 : e <= 16 ? 512 : 384) / threads;
     const int fit = (int)((size_t)228 * 1024 / (z_smem_dbx(tx, L, rb) + 1024));
     const int n = want < fit ? want : fit;
     return e <= 24 && n > 1 ? n : 1;
@@ -1161,7 +1161,11 @@ __device__ __forceinline__ bool z_tile(const Cx<T> *sin, const T *sg, int pr, in
     }
     if (!packed) {
 #pragma unroll
-        for (int m = 0; m < E; ++m) v[m] = cscale(v[m], gval(m) * gscale);
+        for (int m = 0; m < E; ++m) {
+            // the transform left v normalised, and the products enter sums
+            const T s = gval(m) * gscale;
+            v[m] = {rmul(v[m].x, s), rmul(v[m].y, s)};
+        }
     }
 
 #pragma unroll
