@@ -772,6 +772,22 @@ ISOFFT_SHAPE_F32(YShape, 1152, 48, 48, 24)
 ISOFFT_SHAPE_F32(YShape, 1296, 36, 36, 36)
 ISOFFT_SHAPE_F32(YShape, 2048, 32, 32, 32, 2)
 
+// FP64 y lines of 384 and 768 points, 24 points a thread: the passes are bound
+// by FP64 operations, of which radix 24 leaves 4 to 5 % fewer than 12 (a
+// twiddle stage less): K2 + K4 748 + 737 -> 703 + 711 us at 384 x 190 x 100,
+// 238 + 236 -> 225 + 229 at 100 x 384 x 40.  (On 96 and 192 points, and on x
+// rows, the larger tiles cost small meshes more than the operations save.)
+template <>
+struct YShape<double, 384> {
+    static constexpr int E = 24;
+    using Rad = Radices<24, 4, 4>;
+};
+template <>
+struct YShape<double, 768> {
+    static constexpr int E = 24;
+    using Rad = Radices<24, 8, 4>;
+};
+
 // The z pass holds two lines groups per tile and stages its prefetches in
 // shared memory.  512-point FP32 lines run 32 points per thread in two
 // stages (16 32): one exchange per transform instead of two with 8 8 8 (16
