@@ -61,7 +61,7 @@ ISOFFT_HD Cx<T> cfms(Cx<T> a, T r, Cx<T> b) { return {rsub(a.x, rmul(r, b.x)), r
 // 512^3, 34.2 -> 31.4 ms at 1152^3, 64 ragged grids 912 -> 830 us; the x and y
 // passes, bound elsewhere, change by under 3 % either way.  (Float pairs gain
 // nothing: K3 1080 -> 1116 us at 256^3, bound by the lanes.)
-#ifdef __CUDA_ARCH__
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000  // (host checks of this file compile for any architecture)
 ISOFFT_HD Cx<float> packed_fma(Cx<float> b, float r, Cx<float> a)
 {
     const float2 v = __ffma2_rn(make_float2(b.x, b.y), make_float2(r, r), make_float2(a.x, a.y));
