@@ -132,7 +132,8 @@ enum {
  *   stream     stream used for the one-off set-up work (Green's spectrum
  *              build, table uploads); the call synchronises on it before
  *              returning.
- * Allocates the plan's workspace (complex Nz x My x Mx/2) on the current
+ * Allocates the plan's workspace (complex Nz x My x Mx/2, with Nz rounded up
+ * to a multiple of 16 for FP32 meshes of large planes) on the current
  * device and, on a cache miss, the Green's spectrum. */
 int ipf_plan_create(ipf_plan_t *out, const int64_t n[3], const double h[3], int dtype,
                     uint32_t flags, int verbosity, void *stream);

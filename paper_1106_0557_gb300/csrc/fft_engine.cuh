@@ -83,12 +83,6 @@ ISOFFT_HD Cx<T> cmul(Cx<T> a, Cx<T> b)
     return {rsub(rmul(a.x, b.x), rmul(a.y, b.y)), radd(rmul(a.x, b.y), rmul(a.y, b.x))};
 }
 template <typename T>
-ISOFFT_HD Cx<T> cscale(Cx<T> a, T s)
-{
-    a = crenorm(a);
-    return {a.x * s, a.y * s};
-}
-template <typename T>
 ISOFFT_HD Cx<T> cconj(Cx<T> a) { return {a.x, -a.y}; }
 // multiply by -i
 template <typename T>
@@ -870,21 +864,18 @@ ISOFFT_ZSHAPE_F32(1152, 24, 12, 4, 24)
 ISOFFT_ZSHAPE_F32(1536, 24, 8, 8, 24)
 ISOFFT_ZSHAPE_F32(2048, 32, 4, 16, 32)
 #undef ISOFFT_ZSHAPE_F32
-// 16-byte points on 768-point lines (one-column tiles of 128 threads): the
-// radix 12 goes last, where a thread's stage twiddles are shared by all its
-// butterflies (the thread count is a multiple of every stage's stride): 17
-// twiddles a thread instead of 27, and no spills under the 168-register cap
-// (df64 z pass 10.43 -> 9.14 ms at 384^3; the same order at 384 points
-// measured 8 % slower).
-struct ZShape16B768 {
+// FP64 768-point lines (one-column tiles of 128 threads): the radix 12 goes
+// last, where a thread's stage twiddles are shared by all its butterflies (the
+// thread count is a multiple of every stage's stride): 17 twiddles a thread
+// instead of 27 (float pairs, which took these lines too before 1024 points
+// proved faster there: z pass 10.43 -> 9.14 ms at 384^3; the same order at 384
+// points measured 8 % slower).
+template <>
+struct ZShape<double, 768> {
     static constexpr int E = 12;
     using Rad = Radices<4, 4, 4, 12>;
     static constexpr bool TW_REGS = true;
 };
-template <>
-struct ZShape<double, 768> : ZShape16B768 {};
-template <>
-struct ZShape<df64, 768> : ZShape16B768 {};
 // FP64-class 2304-point lines (and FP32 lines of 1296 points, at 36 points a
 // thread: 469 us against 577 at 1536) read their twiddles from the table (a
 // thread's share would not fit in registers next to its points).  FP32 takes

@@ -5,7 +5,8 @@
 // Buffers (C order, x fastest):
 //   src, phi : real [Nz][Ny][Nx]
 //   W        : complex [Nz][My][Kx], Kx = Mx / 2, the plan's workspace (on
-//              2304-point z lines in blocks of 16 planes, w_row below).  The
+//              2304-point z lines, and in FP32 on large planes of z lines of 768
+//              points and more, in blocks of 16 planes, w_row below).  The
 //              z padding is never stored: the z pass reads z < Nz, treats the
 //              rest of its line as zero, and writes back only z < Nz.
 //   G        : real, the transform of the Eq. 9 table on the even octant (it
