@@ -11,9 +11,18 @@
 // One pass per axis transforms every octant line that way in place, with
 // the FFT engine of the solve passes in FP64 (O(M^3 log M) in all); FP64 is
 // what sets the accuracy floor of the solve.
+//
+// A spectrum that is stored in FP32 rounds each bin to 24 bits, so its build
+// takes two cheaper FP64 forms (PAIRS below: inv_sqrt, and two lines per
+// transform).  FP64 and float-pair spectra keep every bit they can: with the
+// cheaper forms FP64 potentials lay further from 80-bit ones, by 3 to 6 % on
+// random sources (at most 1.42 times) and up to 9 times on sources that
+// alternate from cell to cell (36^3 2.7e-15 -> 2.5e-14; allocation-free 4.5e-15
+// -> 8.5e-14), float pairs up to 5 times; FP32 ones did not move.
 #include <math.h>
 #include <stdio.h>
 
+#include <type_traits>
 #include <vector>
 
 #include "launch.h"
@@ -34,7 +43,8 @@ static __device__ __forceinline__ double inv_sqrt(double x)
 
 // A thread takes one (x, y) and `zc` planes; block row blockIdx.y.  Bound by
 // FP64 arithmetic: the quotient by the square root with 64-bit indices took
-// 22.9 us on a 65^3 octant, this 16.8 us (0.82 -> 0.52 ms at 257^3).
+// 22.9 us on a 65^3 octant, PAIRS 16.8 us (0.82 -> 0.52 ms at 257^3).
+template <bool PAIRS>
 static __global__ void k_green_octant(double *__restrict__ g, int X, int Y, int Z, double hx, double hy,
                                       double hz, int zc)
 {
@@ -49,7 +59,15 @@ static __global__ void k_green_octant(double *__restrict__ g, int X, int Y, int 
     for (int z = blockIdx.y * zc; z < z1; ++z) {
         const double dz = hz * (double)z;
         // Eq. 6; at the origin Eq. 9: the largest off-origin magnitude
-        const double v = xy == 0 && z == 0 ? num / hmin : num * inv_sqrt(fma(dz, dz, fma(dx, dx, dy * dy)));
+        double v;
+        if (xy == 0 && z == 0) {
+            v = num / hmin;
+        } else {
+            if constexpr (PAIRS)
+                v = num * inv_sqrt(fma(dz, dz, fma(dx, dx, dy * dy)));
+            else
+                v = num / sqrt(dx * dx + dy * dy + dz * dz);
+        }
         g[(int64_t)z * X * Y + xy] = v;
     }
 }
@@ -57,11 +75,12 @@ static __global__ void k_green_octant(double *__restrict__ g, int X, int Y, int 
 // One axis of the octant transform, in place: line (a, c) of the octant,
 // elements base[q Cc] (q <= L/2, base = oct + a (L/2 + 1) Cc + c), is
 // mirrored to L points, transformed, and bins 0..L/2 (real) are written back.
-// The transform of a real even line is real, so two neighbouring lines go
-// through one complex transform as its real and imaginary parts: the pass is
-// bound by FP64 arithmetic, and this halves it (22.2 -> 15.2 us an axis at
-// 65^3, 1.40 -> 0.82 ms at 257^3).
-// Line pairs are grouped NL per CTA (one row buffer each, as the x passes use).
+// PAIRS (FP32 spectra): the transform of a real even line is real, so two
+// neighbouring lines go through one complex transform as its real and
+// imaginary parts: the pass is bound by FP64 arithmetic, and this halves it
+// (22.2 -> 15.2 us an axis at 65^3, 1.40 -> 0.82 ms at 257^3).  Each line's
+// rounding is then relative to the larger of the two.
+// Lines (or pairs) are grouped NL per CTA (one row buffer each, as the x passes use).
 template <int L>
 struct DctCfg {
     using SH = Shape<double, L>;
@@ -71,7 +90,7 @@ struct DctCfg {
     static constexpr size_t SMEM = (size_t)NL * RowPad<double, L>::LP * sizeof(Cx<double>);
 };
 
-template <int L>
+template <int L, bool PAIRS>
 static __global__ void __launch_bounds__(DctCfg<L>::THREADS)
 k_cos_lines(double *__restrict__ oct, const Cx<double> *__restrict__ tw, int64_t A, int64_t Cc)
 {
@@ -80,11 +99,12 @@ k_cos_lines(double *__restrict__ oct, const Cx<double> *__restrict__ tw, int64_t
     extern __shared__ __align__(16) unsigned char dct_smem[];
     Cx<double> *row = reinterpret_cast<Cx<double> *>(dct_smem) + (threadIdx.x / NT) * RowPad<double, L>::LP;
     const int l = threadIdx.x / NT, t = threadIdx.x % NT;
-    const int64_t lines = A * Cc, pairs = (lines + 1) / 2;
+    constexpr int PER = PAIRS ? 2 : 1;  // lines per transform
+    const int64_t lines = A * Cc, units = (lines + PER - 1) / PER;
     grid_wait();
-    for (int64_t p0 = (int64_t)blockIdx.x * C::NL; p0 < pairs; p0 += (int64_t)gridDim.x * C::NL) {
-        const int64_t line = 2 * (p0 + l);
-        const bool act0 = line < lines, act1 = line + 1 < lines;
+    for (int64_t u0 = (int64_t)blockIdx.x * C::NL; u0 < units; u0 += (int64_t)gridDim.x * C::NL) {
+        const int64_t line = PER * (u0 + l);
+        const bool act0 = line < lines, act1 = PAIRS && line + 1 < lines;
         const int64_t a = act0 ? line / Cc : 0, c = act0 ? line % Cc : 0;
         double *base0 = oct + a * n * Cc + c;
         double *base1 = c + 1 < Cc ? base0 + 1 : oct + (a + 1) * n * Cc;  // line + 1
@@ -110,44 +130,63 @@ k_cos_lines(double *__restrict__ oct, const Cx<double> *__restrict__ tw, int64_t
     }
 }
 
+// the lengths that kMeshLengths (launch.h) gives FP32 only, the 16-byte types
+// only, and both
+#define ISOFFT_DCT_LENGTHS_F32(X) X(324) X(432) X(648) X(1296)
+#define ISOFFT_DCT_LENGTHS_16B(X) X(144)
 #define ISOFFT_DCT_LENGTHS(X) \
-    X(32) X(48) X(64) X(96) X(128) X(144) X(192) X(256) X(288) X(324) X(384) X(432) X(512) X(576) X(648) X(768) \
-    X(1024) X(1152) X(1296) X(1536) X(2048) X(2304)
+    X(32) X(48) X(64) X(96) X(128) X(192) X(256) X(288) X(384) X(512) X(576) X(768) X(1024) X(1152) X(1536) X(2048) \
+    X(2304)
 
-template <int L>
+template <int L, bool PAIRS>
 static cudaError_t run_cos_lines(double *oct, const Cx<double> *tw, int64_t A, int64_t Cc, cudaStream_t st)
 {
     using C = DctCfg<L>;
-    const int64_t groups = ((A * Cc + 1) / 2 + C::NL - 1) / C::NL;
+    const int64_t units = PAIRS ? (A * Cc + 1) / 2 : A * Cc, groups = (units + C::NL - 1) / C::NL;
     const int grid = (int)(groups < 152 * 8 ? groups : 152 * 8);
     if (C::SMEM > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_cos_lines<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+        cudaError_t e =
+            cudaFuncSetAttribute(k_cos_lines<L, PAIRS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
         if (e != cudaSuccess) return e;
     }
-    return launch_pass(k_cos_lines<L>, dim3(grid), C::THREADS, C::SMEM, st, oct, tw, A, Cc);
+    return launch_pass(k_cos_lines<L, PAIRS>, dim3(grid), C::THREADS, C::SMEM, st, oct, tw, A, Cc);
 }
 
 // Cosine transform of every octant line along one axis of length M (one of
 // the supported doubled lengths); tw = W_M^k, k < M.
+template <bool PAIRS>
 static cudaError_t cos_axis(int M, double *oct, const Cx<double> *tw, int64_t A, int64_t Cc, cudaStream_t st)
 {
-    switch (M) {
 #define X_(n) \
-    case n: return run_cos_lines<n>(oct, tw, A, Cc, st);
+    case n: return run_cos_lines<n, PAIRS>(oct, tw, A, Cc, st);
+    switch (M) {
         ISOFFT_DCT_LENGTHS(X_)
-#undef X_
-    default: return cudaErrorInvalidValue;
+    default: break;
     }
+    if constexpr (PAIRS) {
+        switch (M) {
+            ISOFFT_DCT_LENGTHS_F32(X_)
+        default: break;
+        }
+    } else {
+        switch (M) {
+            ISOFFT_DCT_LENGTHS_16B(X_)
+        default: break;
+        }
+    }
+#undef X_
+    return cudaErrorInvalidValue;
 }
 
 // The three axis passes of the octant transform, in place on oct [Z][Y][X];
 // tws[a] = W_{M_a}^k.
+template <bool PAIRS>
 static cudaError_t cos_transform(const int64_t M[3], double *oct, const Cx<double> *const tws[3], cudaStream_t st)
 {
     const int64_t X = M[0] / 2 + 1, Y = M[1] / 2 + 1, Z = M[2] / 2 + 1;
-    cudaError_t e = cos_axis((int)M[0], oct, tws[0], Z * Y, 1, st);
-    if (e == cudaSuccess) e = cos_axis((int)M[1], oct, tws[1], Z, X, st);
-    if (e == cudaSuccess) e = cos_axis((int)M[2], oct, tws[2], 1, X * Y, st);
+    cudaError_t e = cos_axis<PAIRS>((int)M[0], oct, tws[0], Z * Y, 1, st);
+    if (e == cudaSuccess) e = cos_axis<PAIRS>((int)M[1], oct, tws[1], Z, X, st);
+    if (e == cudaSuccess) e = cos_axis<PAIRS>((int)M[2], oct, tws[2], 1, X * Y, st);
     return e;
 }
 
@@ -286,13 +325,14 @@ static cudaError_t spectrum_steps(const int64_t M[3], const double hn[3], T *G, 
     const int X = (int)(M[0] / 2 + 1), Y = (int)(M[1] / 2 + 1), Z = (int)(M[2] / 2 + 1);
     if ((reinterpret_cast<uintptr_t>(tws) & 15) || (reinterpret_cast<uintptr_t>(oct) & 7))
         return cudaErrorMisalignedAddress;  // complex-double tables need 16-byte alignment
+    constexpr bool PAIRS = std::is_same<T, float>::value;
     const int zc = Z > 128 ? 8 : 2;
-    cudaError_t e = launch_pass(k_green_octant, dim3((unsigned)((X * Y + 255) / 256), (unsigned)((Z + zc - 1) / zc)), 256,
+    cudaError_t e = launch_pass(k_green_octant<PAIRS>, dim3((unsigned)((X * Y + 255) / 256), (unsigned)((Z + zc - 1) / zc)), 256,
                                 0, st, oct, X, Y, Z, hn[0], hn[1], hn[2], zc);
     const Cx<double> *tw[3] = {reinterpret_cast<const Cx<double> *>(tws),
                                reinterpret_cast<const Cx<double> *>(tws) + M[0],
                                reinterpret_cast<const Cx<double> *>(tws) + M[0] + M[1]};
-    if (e == cudaSuccess) e = cos_transform(M, oct, tw, st);
+    if (e == cudaSuccess) e = cos_transform<PAIRS>(M, oct, tw, st);
     if (e == cudaSuccess) e = pack_spectrum<T>(M, oct, G, Gs, st);
     return e;
 }
