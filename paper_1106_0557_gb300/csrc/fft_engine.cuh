@@ -263,19 +263,20 @@ struct Dft<T, 3> {
     }
 };
 
-// Float pairs: the sums of the radix 3 stay lazy like the other radices',
-// halving is exact, and the products only enter sums (142 -> 114 FP32
-// operations, against 128 of a radix 4).
+// Float pairs: the generic radix 3 with its halving taken exactly instead of
+// by a product, which gives the same bits (132 FP32 operations for 142,
+// against 128 of a radix 4).  Each sum that enters a product or a second sum
+// is renormalised: with those steps left out (114 operations) the transforms
+// of 24 to 2304 points lay 6 to 8 % further from long double ones.
 template <>
 struct Dft<df64, 3> {
     static ISOFFT_HD void run(Cx<df64> (&a)[3])
     {
         constexpr df64 s3 = (df64)0.8660254037844387;  // sin(2 pi / 3)
-        const Cx<df64> sum = cadd(a[1], a[2]);
-        const Cx<df64> dif = crenorm(csub(a[1], a[2]));  // enters the products
+        const Cx<df64> sum = crenorm(cadd(a[1], a[2])), dif = crenorm(csub(a[1], a[2]));
         const Cx<df64> h = {{-0.5f * sum.x.hi, -0.5f * sum.x.lo}, {-0.5f * sum.y.hi, -0.5f * sum.y.lo}};
-        const Cx<df64> t = cadd(a[0], h);
-        const Cx<df64> u = {rmul(dif.y, s3), -rmul(dif.x, s3)};  // -i s3 (a1 - a2)
+        const Cx<df64> t = crenorm(cadd(a[0], h));
+        const Cx<df64> u = {dif.y * s3, -(dif.x * s3)};  // -i s3 (a1 - a2)
         a[0] = cadd(a[0], sum);
         a[1] = cadd(t, u);
         a[2] = csub(t, u);
