@@ -24,10 +24,10 @@ namespace isofft {
 //            lines);
 //   FP32 x:  432 31 + 33 against 22 + 23 at 512: left out; elsewhere a few
 //            per cent on the x passes buy 9 to 16 % fewer columns;
-//   df64 z:  lines of powers of two hold more warps and no radix 3: 192 68,
-//            288 131, 512 152, 576 299, 1024 340, 1152 501, 1536 787, 2048 908,
-//            2304 1406; with a radix 3 of fewer roundings, which was not kept,
-//            144 took 69 (192: 69), 384 194 and 768 401, so those are not
+//   df64 z:  lines of powers of two hold more warps and no radix 3: 192 70,
+//            288 126, 512 154, 576 302, 1024 344, 1152 522, 1536 876, 2048 913,
+//            2304 1467; with fewer roundings, which were not kept, 144 took 69
+//            (192: 69), 384 194 and 768 401, so those are not
 //            taken on z, and 324 319, 432 226 and 648 658, so those on no axis;
 //   FP64 z:  144 220, 192 303, 288 509, 324 742, 384 673, 576 1112, 648 1550,
 //            768 1457, 1152 2455, 1296 3375, 1536 3373, 2048 4284, 2304 5416.

@@ -1162,11 +1162,7 @@ __device__ __forceinline__ bool z_tile(const Cx<T> *sin, const T *sg, int pr, in
     }
     if (!packed) {
 #pragma unroll
-        for (int m = 0; m < E; ++m) {
-            // the transform left v normalised, and the products enter sums
-            const T s = gval(m) * gscale;
-            v[m] = {rmul(v[m].x, s), rmul(v[m].y, s)};
-        }
+        for (int m = 0; m < E; ++m) v[m] = cscale(v[m], gval(m) * gscale);
     }
 
 #pragma unroll

@@ -1,8 +1,10 @@
-// df64_radix3_check.cu -- the float-pair radix 3 of fft_engine.cuh on the CPU
-// against its definition in normalised float-pair arithmetic (operators of
-// df64.cuh), on normalised and lazily summed inputs of random magnitudes.
-// Built and run by tests/test_df64_radix3_host.py.  Prints the number of
-// values and of values that differ in any bit.
+// df64_rounding_check.cu -- the float-pair radix 3 and the product with the
+// spectrum (fft_engine.cuh) on the CPU: the radix 3 against its definition in
+// normalised float-pair arithmetic (operators of df64.cuh), on normalised and
+// lazily summed inputs of random magnitudes; the product for results that are
+// normalised (adding the parts again changes neither).
+// Built and run by tests/test_df64_rounding_host.py.  Prints, for each, the
+// number of values and of those that fail.
 #include <math.h>
 #include <stdio.h>
 
@@ -39,6 +41,15 @@ int main()
             for (int c = 0; c < 2; ++c, ++n) bad += got[c].hi != want[c].hi || got[c].lo != want[c].lo;
         }
     }
-    printf("%ld %ld\n", n, bad);
+    printf("radix3 %ld %ld\n", n, bad);
+    n = bad = 0;
+    for (long i = 0; i < 1000000; ++i) {
+        const Cx<df64> v = cscale(Cx<df64>{df64(rnd()), df64(rnd())}, df64(rnd()));
+        const Cx<df64> w = norm(v);
+        n += 2;
+        bad += v.x.hi != w.x.hi || v.x.lo != w.x.lo;
+        bad += v.y.hi != w.y.hi || v.y.lo != w.y.lo;
+    }
+    printf("product %ld %ld\n", n, bad);
     return 0;
 }
