@@ -70,6 +70,7 @@ inline cudaError_t launch_pass(void (*kernel)(K...), dim3 grid, int threads, siz
     cfg.attrs = at;
     cfg.numAttrs = 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, K(args)...);
+    if (e != cudaSuccess) cudaGetLastError();  // reported here; not left for the caller's next check
     count_launch();
     return e;
 }
