@@ -240,44 +240,20 @@ template size_t spectrum_elems<df64>(const int64_t *);
 
 void host_roots(int64_t n, int64_t count, double *re, double *im)
 {
-    // e^{-2 pi i k/n}: reduce k to [0, n/8] by the exact symmetries of the
-    // circle (n is a multiple of 4 for every length used here; other n fall
-    // back to the direct angle).
+    // e^{-2 pi i k/n}: the angle, in units of 2 pi / (4 n), is reduced to the
+    // first octant by the exact symmetries of the circle.
     for (int64_t k = 0; k < count; ++k) {
-        int64_t r = ((k % n) + n) % n;
-        double c, s;  // cos and sin of 2 pi r / n
-        if (n % 4 == 0) {
-            bool neg_s = false;
-            if (2 * r > n) {  // lower half: sin negative
-                r = n - r;
-                neg_s = true;
-            }
-            // r in [0, n/2]
-            bool neg_c = false;
-            if (4 * r > n) {  // second quadrant: cos(pi - a) = -cos a, sin same
-                r = n / 2 - r;
-                neg_c = true;
-            }
-            // r in [0, n/4]
-            double cc, ss;
-            if (8 * r > n) {  // past n/8: swap cos and sin of the complement
-                const double a = 2.0 * M_PI * (double)(n / 4 - r) / (double)n;
-                cc = sin(a);
-                ss = cos(a);
-            } else {
-                const double a = 2.0 * M_PI * (double)r / (double)n;
-                cc = cos(a);
-                ss = sin(a);
-            }
-            c = neg_c ? -cc : cc;
-            s = neg_s ? -ss : ss;
-        } else {
-            const double a = 2.0 * M_PI * (double)r / (double)n;
-            c = cos(a);
-            s = sin(a);
-        }
-        re[k] = c;
-        im[k] = -s;
+        int64_t u = 4 * (((k % n) + n) % n);
+        const bool neg_s = u > 2 * n;  // lower half: sin negative
+        if (neg_s) u = 4 * n - u;
+        const bool neg_c = u > n;  // second quadrant: cos(pi - a) = -cos a, sin same
+        if (neg_c) u = 2 * n - u;
+        const bool swap = 2 * u > n;  // past the octant: cos and sin of the complement
+        if (swap) u = n - u;
+        const double a = 2.0 * M_PI * (double)u / (double)(4 * n);
+        const double c = swap ? sin(a) : cos(a), s = swap ? cos(a) : sin(a);
+        re[k] = neg_c ? -c : c;
+        im[k] = neg_s ? s : -s;
     }
 }
 
