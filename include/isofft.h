@@ -277,7 +277,9 @@ int ipf_plan_pass_times(ipf_plan_t plan, float ms[5]);
  * and keeps the fastest per pass; the choice is remembered per (dtype, mesh,
  * shape, device) for the process, and in the file named by the environment
  * variable ISOFFT_TUNE_FILE if set (read at the first plan, rewritten as
- * choices are made).  ISOFFT_TUNE=0 skips the timing and takes the built-in
+ * choices are made; a file that does not name the digest of this library's
+ * pass code is ignored, since its choices were timed on other kernels).
+ * ISOFFT_TUNE=0 skips the timing and takes the built-in
  * rule (streamed for FP32 lines of 512 to 1024 points, tiles elsewhere).
  * Not in the paper: the tuning of this implementation's tile shapes. */
 int ipf_plan_variants(const ipf_plan_t plan, int v[2]);

@@ -23,20 +23,33 @@ FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "--expt-relaxe
          "-I", INCLUDE, "-I", CSRC]
 
 
-def _spectrum_code():
-    """32-bit digest of the sources that define the cached Green's spectrum
-    (its build and layout); spectrum files written by other code are
-    rejected (see ISOFFT_SPECTRUM_DIR in include/isofft.h)."""
+def _digest(*sources):
+    """32-bit digest of source files, never zero."""
     import hashlib
     h = hashlib.sha256()
-    for fn in ("greens.cu", "launch.h", "fft_engine.cuh", "passes.cuh"):
+    for fn in sources:
         with open(os.path.join(CSRC, fn), "rb") as f:
             h.update(f.read())
     return "0x%08x" % (int(h.hexdigest()[:8], 16) | 1)
 
 
+def _spectrum_code():
+    """Digest of the sources that define the cached Green's spectrum (its build
+    and layout); spectrum files written by other code are rejected (see
+    ISOFFT_SPECTRUM_DIR in include/isofft.h)."""
+    return _digest("greens.cu", "launch.h", "fft_engine.cuh", "passes.cuh")
+
+
+def _pass_code():
+    """Digest of the sources that define the timed y passes and the workspace
+    they run on; timed forms written by other code are rejected (see
+    ISOFFT_TUNE_FILE in include/isofft.h)."""
+    return _digest("passes_inst.cu", "passes.cuh", "fft_engine.cuh", "df64.cuh", "tma.cuh", "launch.h", "api.cu")
+
+
 def _units():
-    units = [("api", "api.cu", ["-DISOFFT_SPECTRUM_CODE=%s" % _spectrum_code()]), ("greens", "greens.cu", []),
+    codes = ["-DISOFFT_SPECTRUM_CODE=%s" % _spectrum_code(), "-DISOFFT_PASS_CODE=%s" % _pass_code()]
+    units = [("api", "api.cu", codes), ("greens", "greens.cu", []),
              ("noalloc", "noalloc.cu", []), ("batch", "batch.cu", [])]
     for real, tag, num in (("isofft::df64", "df64", 3), ("float", "f32", 1), ("double", "f64", 2)):
         for group, gname in ((2, "y"), (3, "z"), (1, "x")):

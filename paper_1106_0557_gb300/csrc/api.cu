@@ -25,6 +25,7 @@
 
 #include "../../include/isofft.h"
 #include "launch.h"
+#include "tune_file.h"
 
 namespace isofft {
 
@@ -299,64 +300,28 @@ int read_status(ipf_plan_s *p, cudaStream_t st)
 // y-pass form tuning: the three forms (tiles, streamed, half-width tiles)
 // run a few times each on the plan's workspace and the fastest is kept per
 // direction, per (dtype, My, Kx, Ny, Nz, device capability); the choices
-// persist for the process and, with ISOFFT_TUNE_FILE, in a JSON file of
-// entries [dtype, My, Kx, Ny, Nz, sm, forward, inverse].
+// persist for the process and, with ISOFFT_TUNE_FILE, in a JSON file
+// (tune_file.h).
 // ---------------------------------------------------------------------
-struct TuneKey {
-    int v[6];
-    bool operator<(const TuneKey &o) const { return std::lexicographical_compare(v, v + 6, o.v, o.v + 6); }
-};
 std::mutex g_tune_mu;
-std::map<TuneKey, std::pair<int, int>> g_tune;
+TuneMap g_tune;
 bool g_tune_loaded = false;
+
+#ifndef ISOFFT_PASS_CODE
+#error "the build passes ISOFFT_PASS_CODE (a digest of the pass code)"
+#endif
 
 void tune_file_load()
 {
     g_tune_loaded = true;
     const char *path = getenv("ISOFFT_TUNE_FILE");
-    if (!path || !path[0]) return;
-    FILE *f = fopen(path, "r");
-    if (!f) return;
-    // the integers of the file in order, eight per entry
-    std::vector<long> nums;
-    long cur = 0;
-    bool in = false, neg = false;
-    for (int ch; (ch = fgetc(f)) != EOF;) {
-        if (ch >= '0' && ch <= '9') {
-            cur = cur * 10 + (ch - '0');
-            in = true;
-        } else {
-            if (in) nums.push_back(neg ? -cur : cur);
-            neg = ch == '-';
-            cur = 0;
-            in = false;
-        }
-    }
-    if (in) nums.push_back(neg ? -cur : cur);
-    fclose(f);
-    for (size_t i = 0; i + 8 <= nums.size(); i += 8) {
-        TuneKey k;
-        for (int j = 0; j < 6; ++j) k.v[j] = (int)nums[i + j];
-        const int a = (int)nums[i + 6], b = (int)nums[i + 7];
-        if (a >= 0 && a < kYForms && b >= 0 && b < kYForms) g_tune[k] = {a, b};
-    }
+    if (path && path[0]) tune_file_read(path, ISOFFT_PASS_CODE, kYForms, g_tune);
 }
 
 void tune_file_save()
 {
     const char *path = getenv("ISOFFT_TUNE_FILE");
-    if (!path || !path[0]) return;
-    FILE *f = fopen(path, "w");
-    if (!f) return;
-    fprintf(f, "{\"y_pass_forms\": [\n");
-    size_t i = 0;
-    for (const auto &kv : g_tune) {
-        const int *v = kv.first.v;
-        fprintf(f, "  [%d, %d, %d, %d, %d, %d, %d, %d]%s\n", v[0], v[1], v[2], v[3], v[4], v[5], kv.second.first,
-                kv.second.second, ++i < g_tune.size() ? "," : "");
-    }
-    fprintf(f, "]}\n");
-    fclose(f);
+    if (path && path[0]) tune_file_write(path, ISOFFT_PASS_CODE, g_tune);
 }
 
 // Mean device milliseconds of three launches after one warm-up.
