@@ -47,8 +47,16 @@ namespace isofft {
 
 // Launch with the programmatic-serialization attribute: the launch is
 // processed while the stream's previous kernel still runs, its CTAs start as
-// that kernel's last ones leave, and each waits in grid_wait() before it
-// touches the previous results.  Without it every pass of a small solve paid
+// that kernel's last ones leave.  Two rules keep that sound:
+//  - every CTA of every kernel launched here passes grid_wait() before it
+//    leaves, also where it has nothing to do or gives up;
+//  - before grid_wait() a kernel writes no global memory and reads only what a
+//    kernel at least two launches back, or a completed copy, has written (the
+//    root tables: in the allocation-free chain k_tables writes them, and the
+//    spectrum's kernels lie between it and the passes).  A CTA starts once the
+//    previous kernel's CTAs have left, hence passed their wait: all before
+//    that kernel is complete and visible, that kernel's own writes are not.
+// Without the attribute every pass of a small solve paid
 // about 2 us between kernels: solves back to back in one stream took 24.9 us
 // at FP32 64^3 (17.2 now), 28.0 at 100 x 70 x 30 (17.7), 70.0 at 128^3 (57.0),
 // 416 at 256^3 (404.5).  The kernels do not trigger their successors early

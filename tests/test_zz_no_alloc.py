@@ -36,10 +36,10 @@ def test_noalloc_matches_plan_solve_on_consecutive_calls(dtype, oracle_mod):
         pytest.skip("no CUDA device")
     from paper_1106_0557_gb300 import Plan
     stream = torch.cuda.current_stream().cuda_stream
-    # (16, 300, 16): 768-point y lines, which FP32 runs in the streamed y form
+    # (16, 330, 16): 768-point y lines, which FP32 runs in the streamed y form
     # (tensor maps over the static array); the others take the tile form
     cases = [((40, 33, 24), (1.0, 1.0, 1.0), 1), ((32, 20, 17), (0.5, 0.25, 1.0), 2),
-             ((40, 33, 24), (1.0, 1.0, 1.0), 3), ((16, 300, 16), (1.0, 0.5, 1.0), 4)]
+             ((40, 33, 24), (1.0, 1.0, 1.0), 3), ((16, 330, 16), (1.0, 0.5, 1.0), 4)]
     for N, h, seed in cases:
         src = _src(N, seed, dtype)
         got = torch.empty_like(src)
@@ -53,6 +53,46 @@ def test_noalloc_matches_plan_solve_on_consecutive_calls(dtype, oracle_mod):
         want = oracle_mod.solve(src.double().cpu().numpy(), h)
         err = oracle_mod.max_rel_error(got.double().cpu().numpy(), want)
         assert err <= TOL[dtype], (N, h, dtype, err)
+
+
+def test_noalloc_calls_in_flight_share_the_scratch_in_order():
+    """Every call rewrites the shared tables and workspace, and its first
+    kernels are launched while the previous call's last pass drains; the
+    transform passes read the tables before they wait for their predecessor.
+    Calls of other meshes and dtypes in turn, with no synchronisation between
+    them, give bitwise what each gives alone."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1106_0557_gb300 import Plan
+    stream = torch.cuda.current_stream().cuda_stream
+    # x lengths of 384 and 768 load the rows' roots before they wait, every z
+    # line its own; 324 is a length of FP32 alone, 144 and 288 of FP64; small
+    # meshes follow one another most closely
+    cases = [((190, 10, 12), "f32"), ((9, 20, 15), "f64"), ((380, 8, 9), "f32"), ((160, 10, 9), "f32"),
+             ((8, 8, 8), "f32"), ((70, 12, 30), "f64"), ((16, 330, 16), "f32"), ((12, 10, 140), "f64"),
+             ((50, 60, 40), "f32"), ((16, 16, 16), "f64")]
+    h = (1.0, 0.5, 0.75)
+    srcs = [_src(N, i, dtype) for i, (N, dtype) in enumerate(cases)]
+
+    def call(i, out):
+        native.ipf_solve_noalloc(cases[i][0], h, cases[i][1], srcs[i].data_ptr(), out.data_ptr(), stream)
+
+    want = [torch.empty_like(s) for s in srcs]
+    for i, (N, dtype) in enumerate(cases):
+        torch.cuda.synchronize()
+        call(i, want[i])
+        torch.cuda.synchronize()
+        with Plan(N, h, dtype, flags=native.IPF_FLAG_PASS_EVENTS) as p:  # its passes do not overlap
+            assert _rel(want[i], p.solve(srcs[i])) <= TOL[dtype], cases[i]
+    order = list(range(len(cases))) + list(range(len(cases)))[::-1] + [0, 4, 2, 4, 0, 9, 2, 9, 6, 3, 6]
+    for _ in range(3):
+        outs = [torch.zeros_like(srcs[i]) for i in order]
+        torch.cuda.synchronize()
+        for i, o in zip(order, outs):
+            call(i, o)
+        torch.cuda.synchronize()
+        assert all(torch.equal(o, want[i]) for i, o in zip(order, outs))
+    native.ipf_noalloc_check(stream)
 
 
 def test_noalloc_rejects_oversize_and_bad_arguments():
