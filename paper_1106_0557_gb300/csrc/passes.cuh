@@ -94,7 +94,8 @@ __host__ __device__ __forceinline__ size_t w_row(int64_t z, int64_t y, int64_t M
     return (size_t)((((z >> zsh) * My + y) << zsh) + (z & ((int64_t(1) << zsh) - 1)));
 }
 // (A z-blocked workspace is allocated in whole blocks; its last block may hold
-// planes past the mesh, which no pass writes and the z pass masks.)
+// planes past the mesh, which the z pass masks where it reads them and may
+// overwrite where it stores whole boxes, and no other pass touches.)
 inline int64_t w_blocks(int64_t nz, int zsh) { return (nz + (int64_t(1) << zsh) - 1) >> zsh; }
 
 // Asynchronous global -> shared copies (cp.async): BYTES = 4, 8 or 16;
