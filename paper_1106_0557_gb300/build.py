@@ -37,7 +37,7 @@ def _spectrum_code():
     """Digest of the sources that define the cached Green's spectrum (its build
     and layout); spectrum files written by other code are rejected (see
     ISOFFT_SPECTRUM_DIR in include/isofft.h)."""
-    return _digest("greens.cu", "launch.h", "fft_engine.cuh", "passes.cuh")
+    return _digest("greens.cu", "inv_sqrt.cuh", "launch.h", "fft_engine.cuh", "passes.cuh")
 
 
 def _pass_code():
