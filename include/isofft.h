@@ -119,10 +119,13 @@ enum {
  *              512, 768, 1024, 1536, 2304 or, where the axis and dtype have
  *              a faster pass of that length, 144, 288, 324, 432, 576, 648,
  *              1152, 1296, 2048) must fit the largest supported length, else
- *              IPF_UNSUPPORTED_SIZE; ipf_plan_padded_shape tells it.  1152^3 cells in FP32 need
- *              about 37 GB of device memory: a 24.5 GB workspace and a 6 GB
- *              spectrum, plus 24.5 GB of FP64 scratch while the spectrum is
- *              built.
+ *              IPF_UNSUPPORTED_SIZE; ipf_plan_padded_shape tells it.  1152^3
+ *              cells in FP32 need about 31 GB of device memory, a 24.5 GB
+ *              workspace and a 6 GB spectrum, plus 12.3 GB of FP64 scratch
+ *              while the spectrum is built.  IPF_DF64 plans take 512 and 1024
+ *              points on z, not 384 and 768 (N_z of 145 to 192 and of 289 to
+ *              384): faster, at a third more memory for the spectrum and its
+ *              scratch.
  *   h          {hx, hy, hz}, each finite and > 0.
  *   dtype      IPF_F32, IPF_F64 or IPF_DF64.  The Green's spectrum is always
  *              built in FP64 and rounded to the plan's dtype.

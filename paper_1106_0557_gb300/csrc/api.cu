@@ -177,14 +177,15 @@ struct ipf_plan_s {
 namespace {
 
 // z blocking of the workspace (w_row): where the z pass copies rows of 32 or
-// 16 bytes (lines of 768 points and more), one row per plane, and the planes
+// 16 bytes (FP32 lines of 768 points and more), one row per plane, and the planes
 // are so large that each row lies in a memory page of its own (2 MB).  In
 // blocks of 16 planes the rows of a line come from 16 times fewer pages: K3
 // 2373 -> 1612 us at FP32 768 x 384 x 384 (planes of 4.7 MB), 2730 -> 1572 at
 // 512^3, 924 -> 813 at 384^3 (2.4 MB); at 309^3 (1.7 MB) 566 -> 590, and on
 // planes of 1 MB and less the solve is no faster (366 -> 369 us at
-// 256 x 128 x 384), so those stay plain.  2304-point lines of whole blocks
-// take them for every dtype and plane.
+// 256 x 128 x 384), so those stay plain.  Lines of 1296 points stay plain too
+// (their boxes of 216 planes are not whole blocks): 580^3, planes of 6.7 MB, takes
+// 10.0 ms.  2304-point lines of whole blocks take them for every dtype and plane.
 int plan_zsh(const int64_t M[3], int64_t Nz, int dtype)
 {
     if (M[2] == 2304 && Nz % (1 << kZBlockShift) == 0) return kZBlockShift;

@@ -42,7 +42,8 @@ constexpr MeshLength kMeshLengths[] = {
     {512, {7, 7, 7}},  {576, {7, 7, 7}},  {648, {3, 0, 0}},  {768, {7, 7, 3}},  {1024, {7, 7, 7}}, {1152, {7, 7, 7}},
     {1296, {7, 0, 0}}, {1536, {7, 7, 7}}, {2048, {7, 7, 7}}, {2304, {7, 7, 7}}};
 constexpr int kMaxM = 2304;
-// Whether z lines of length Mz have an instance on a z-blocked workspace.
+// Whether z lines of length Mz have an instance on a z-blocked workspace (1296
+// points would need blocks of 8 planes or less).
 constexpr bool z_blocks(int Mz, bool f32)
 {
     return Mz == 2304 || (f32 && (Mz == 768 || Mz == 1024 || Mz == 1152 || Mz == 1536 || Mz == 2048));

@@ -5,9 +5,9 @@
 // Buffers (C order, x fastest):
 //   src, phi : real [Nz][Ny][Nx]
 //   W        : complex [Nz][My][Kx], Kx = Mx / 2, the plan's workspace (on
-//              2304-point z lines, and in FP32 on large planes of z lines of 768
-//              points and more, in blocks of 16 planes, w_row below).  The
-//              z padding is never stored: the z pass reads z < Nz, treats the
+//              2304-point z lines of whole blocks, and in FP32 on planes of 2 MB
+//              and more of z lines of 768 points and more but 1296, in blocks
+//              of 16 planes, w_row below).  The z padding is never stored: the z pass reads z < Nz, treats the
 //              rest of its line as zero, and writes back only z < Nz.
 //   G        : real, the transform of the Eq. 9 table on the even octant (it
 //              is real and even in every axis) in the tiled order of
@@ -375,11 +375,12 @@ struct ZCfg {
     // instead of two; the input is then staged once per tile (the next
     // tile's copies start after the first exchange's barrier, when every
     // thread has read its input).  Taken wherever the extra buffer fits the
-    // CTAs per SM (k_z_convolve; every length but 2304) and the tiles are
-    // wider than one 16-byte column.  Otherwise one exchange buffer and an
-    // input set twice as wide (k_z_convolve_pairs: 2304-point lines, and the
-    // 768-point lines of 16-byte points, 6.93 -> 6.62 ms for a df64 384^3
-    // solve's z pass).
+    // CTAs per SM and the tiles are wider than one 16-byte column
+    // (k_z_convolve).  Otherwise one exchange buffer and an input set twice as
+    // wide (k_z_convolve_pairs: FP32 lines of 1296, 2048 and 2304 points;
+    // 16-byte points on lines of 576, 768, 1536, 2048 and 2304, where a float-
+    // pair 384^3 z pass on 768-point lines went from 6.93 to 6.62 ms before
+    // 1024 points took its place).
     static constexpr size_t SMEM_DBX =
         2 * XCH + (size_t)2 * boxes(SHIFT_FITS) * box_rows(SHIFT_FITS) * TX * sizeof(Cx<T>) + 2 * G_SET + 16 + TWS;
     // tiles with 16-byte copy rows (16-byte points on 1-column tiles, the
@@ -758,7 +759,7 @@ k_x_forward(const In<T> *__restrict__ src, Cx<T> *__restrict__ W, const Cx<T> *_
         RowTwiddles<true, T, L, SH> twr;
         twr.load(tw, t);
         grid_wait();
-            for (int64_t r0 = (int64_t)blockIdx.x * C::NL; r0 < nrows; r0 += (int64_t)gridDim.x * C::NL) {
+        for (int64_t r0 = (int64_t)blockIdx.x * C::NL; r0 < nrows; r0 += (int64_t)gridDim.x * C::NL) {
             const int64_t row = r0 + l;  // row = z * Ny + y
             const bool active = row < nrows;
             x_forward_row<T, L, true, SH>(src, W, tw, rtw, Nx, Ny, My, active ? row : 0, active, line, t, zsh, twr);
@@ -773,7 +774,7 @@ k_x_forward(const In<T> *__restrict__ src, Cx<T> *__restrict__ W, const Cx<T> *_
         const int64_t row = (int64_t)blockIdx.x * C::NL + l;
         const bool active = row < nrows;
         x_forward_row<T, L, false, SH>(src, W, tw, rtw, Nx, Ny, My, active ? row : 0, active, line, t, zsh);
-        }
+    }
 }
 
 template <typename T, int L>
@@ -789,7 +790,7 @@ k_x_inverse(const Cx<T> *__restrict__ W, In<T> *__restrict__ phi, const Cx<T> *_
         RowTwiddles<true, T, L> twr;
         twr.load(tw, t);
         grid_wait();
-            for (int64_t r0 = (int64_t)blockIdx.x * C::NL; r0 < nrows; r0 += (int64_t)gridDim.x * C::NL) {
+        for (int64_t r0 = (int64_t)blockIdx.x * C::NL; r0 < nrows; r0 += (int64_t)gridDim.x * C::NL) {
             const int64_t row = r0 + l;
             const bool active = row < nrows;
             x_inverse_row<T, L, false, true>(W, phi, tw, rtw, Nx, Ny, My, active ? row : 0, active, line, t, zsh,
@@ -800,7 +801,7 @@ k_x_inverse(const Cx<T> *__restrict__ W, In<T> *__restrict__ phi, const Cx<T> *_
         const int64_t row = (int64_t)blockIdx.x * C::NL + l;
         const bool active = row < nrows;
         x_inverse_row<T, L>(W, phi, tw, rtw, Nx, Ny, My, active ? row : 0, active, line, t, zsh);
-        }
+    }
 }
 
 // ---------------------------------------------------------------------
