@@ -59,7 +59,7 @@ ISOFFT_HD Cx<T> cfms(Cx<T> a, T r, Cx<T> b) { return {rsub(a.x, rmul(r, b.x)), r
 // roundings; the FP32 lanes take two cycles, but the issue slot is one, and
 // the z pass is bound by issue).  K3 189 -> 178.5 us at 256^3, 1570 -> 1491 at
 // 512^3, 34.2 -> 31.4 ms at 1152^3, 64 ragged grids 912 -> 830 us; the x and y
-// passes, bound elsewhere, change by under 3 % either way.  (Float pairs gain
+// passes, bound elsewhere, take 1 to 4 % longer (K2 73.0 -> 75.7 at 256^3).  (Float pairs gain
 // nothing: K3 1080 -> 1116 us at 256^3, bound by the lanes.)
 #if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000  // (host checks of this file compile for any architecture)
 ISOFFT_HD Cx<float> packed_fma(Cx<float> b, float r, Cx<float> a)
